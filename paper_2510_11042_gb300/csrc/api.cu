@@ -127,13 +127,18 @@ static int cuda_fail(lbem_ctx *h, cudaError_t e, const char *what)
     } while (0)
 
 // Kernel status word: a step kernel that gave up on a bounded wait sets bit 0.
+static int step_status(lbem_ctx *h, int st)
+{
+    if (st & 1) return fail(h, LBEM_ERR_TIMEOUT, "a step kernel gave up waiting for its staged copies");
+    return LBEM_OK;
+}
+
 static int check_status(lbem_ctx *h)
 {
     int st = 0;
     CK(h, cudaMemcpyAsync(&st, h->flag + 1, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
-    if (st & 1) return fail(h, LBEM_ERR_TIMEOUT, "a step kernel gave up waiting for its staged copies");
-    return LBEM_OK;
+    return step_status(h, st);
 }
 
 // In-place streaming: bring the state to the canonical layout (after a push
@@ -1646,15 +1651,18 @@ int32_t lbem_probe(lbem_handle h, const int32_t *xyz, int32_t n, float *out)
 int32_t lbem_fields(lbem_handle h, float *E, float *H, int32_t on_device)
 {
     if (!h || !E || !H) return fail(h, LBEM_ERR_ARG, "NULL argument");
-    for (int comp = 0; comp < 6; ++comp) {
-        float *dst = (comp < 3 ? E : H) + (size_t)(comp % 3) * h->ncell;
-        float *out = on_device ? dst : h->stage;
-        AA_SETTLE(h);
+    // device maps in one launch; host maps one component at a time through the staging plane
+    AA_SETTLE(h);
+    float *dst[6];
+    for (int comp = 0; comp < 6; ++comp) dst[comp] = (comp < 3 ? E : H) + (size_t)(comp % 3) * h->ncell;
+    for (int comp = 0; comp < (on_device ? 1 : 6); ++comp) {
+        float *one[6] = {};
+        one[comp] = h->stage;
         CK(h, launch_fields(h->g.mode, h->g.storage, h->f[h->cur], h->inv_eps, h->mu_on ? h->inv_mu : nullptr, h->scale, h->P,
-                            h->g.nx, h->g.ny, h->g.nz, h->nxp, inc_view(h), comp, out, h->stream));
+                            h->g.nx, h->g.ny, h->g.nz, h->nxp, inc_view(h), on_device ? dst : one, h->stream));
         h->launches += 1;
         if (!on_device) {
-            CK(h, cudaMemcpyAsync(dst, h->stage, (size_t)h->ncell * 4, cudaMemcpyDeviceToHost, h->stream));
+            CK(h, cudaMemcpyAsync(dst[comp], h->stage, (size_t)h->ncell * 4, cudaMemcpyDeviceToHost, h->stream));
             CK(h, cudaStreamSynchronize(h->stream));
         }
     }
@@ -1687,13 +1695,15 @@ int32_t lbem_energy(lbem_handle h, double *out)
     int l = 0;
     AA_SETTLE(h);
     CK(h, launch_energy(h->g.mode, h->g.storage, h->f[h->cur], h->inv_eps, h->mu_on ? h->inv_mu : nullptr, h->scale, h->P, h->g.nx,
-                        h->g.ny, h->g.nz, h->nxp, inc_view(h), part, (int)(h->scratch_doubles - 8),
-                        d_out, h->stream, &l));
+                        h->g.ny, h->nxp, inc_view(h), part, (int)(h->scratch_doubles - 8), h->flag + 1, d_out,
+                        h->stream, &l));
     h->launches += l;
-    CK(h, cudaMemcpyAsync(out, d_out, 8, cudaMemcpyDeviceToHost, h->stream));
+    double got[2];
+    CK(h, cudaMemcpyAsync(got, d_out, sizeof got, cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
+    *out = got[0];
     if (!std::isfinite(*out)) return fail(h, LBEM_ERR_NONFINITE, "non-finite population in the state");
-    return check_status(h);
+    return step_status(h, (int)got[1]);
 }
 
 // checkpoint: header | populations | incident line | line DFT | face DFT

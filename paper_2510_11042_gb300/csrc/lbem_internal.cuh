@@ -410,13 +410,14 @@ cudaError_t launch_add_incident(int mode, int storage, void *f, long long P, int
                                 cudaStream_t s);
 cudaError_t launch_probe(int mode, int storage, const void *f, float scale, long long P, int ny, int nxp,
                          const int *xyz, int n, const IncView &inc, float *out, cudaStream_t s);
+// out: E_x..E_z, H_x..H_z maps (null: not wanted), one pass over the populations
 cudaError_t launch_fields(int mode, int storage, const void *f, const float *inv_eps, const float *inv_mu,
                           float scale, long long P, int nx, int ny, int nz, int nxp,
-                          const IncView &inc, int comp, float *out, cudaStream_t s);
+                          const IncView &inc, float *const out[6], cudaStream_t s);
+// out[0]: the energy, out[1]: the kernel status word
 cudaError_t launch_energy(int mode, int storage, const void *f, const float *inv_eps, const float *inv_mu,
-                          float scale, long long P, int nx, int ny, int nz, int nxp,
-                          const IncView &inc, double *partial, int max_partial, double *out,
-                          cudaStream_t s, int *launches);
+                          float scale, long long P, int nx, int ny, int nxp, const IncView &inc, double *partial,
+                          int max_partial, const int *status, double *out, cudaStream_t s, int *launches);
 
 // ---------------------------------------------------------------- adjoint
 // One backward step of the discrete adjoint (adjoint.cu).  lin_q holds

@@ -9,7 +9,7 @@
 #include <mutex>
 #include <type_traits>
 
-#include "lbem_internal.cuh"
+#include "step_cell.cuh"
 
 namespace lbem {
 namespace {
@@ -475,60 +475,113 @@ static cudaError_t probe_t(const void *f, float sc, long long P, int ny, int nxp
 }
 
 // ------------------------------------------------------------ fields & energy
+// D and B of the total field of the cell at (x, y, z), element c of a padded
+// plane: the populations by vector loads of whole groups (a scalar load per
+// population fetched every sector of a group two or four times, which with
+// 64-bit divides held the old kernels at a tenth of the copy bandwidth), each
+// population scaled and completed by its incident part before it is summed in
+// direction order.  The closed-form wave is evaluated once per cell.
 template <int MODE, class S>
-__device__ __forceinline__ void cell_DB(const S *f, float sc, long long P, long long c,
-                                        const IncView &inc, int x, int y, int z, float D[3],
-                                        float B[3])
+__device__ __forceinline__ void cell_DB(const S *f, float sc, long long P, int c, const IncView &inc, int x, int y,
+                                        int z, float D[3], float B[3])
 {
     using PL = Planes<MODE>;
+    using M = Mode<MODE>;
+    constexpr int NC = PL::NC, NE = PL::NE;
+    const bool in = inc.on && in_box(x, y, z, inc.tf_lo, inc.tf_hi);
+    float E0[3] = {0.f, 0.f, 0.f}, H0[3] = {0.f, 0.f, 0.f};
+    if (in && inc.on == 2) {
+        const float amp = (float)pw_amplitude(inc.pw, x, y, z, inc.t);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            E0[k] = amp * (float)inc.pw.pol[k];
+            H0[k] = amp * (float)inc.pw.kxp[k];
+        }
+    }
+    const int sl = inc.axis == 0 ? x : (inc.axis == 1 ? y : z);
     D[0] = D[1] = D[2] = 0.f;
     B[0] = B[1] = B[2] = 0.f;
 #pragma unroll
-    for (int q = 0; q < PL::Q; ++q) {
-        const float v = ldv<S>(f + pop_index(MODE, (int)sizeof(S), P, q, c)) * sc + inc_at(inc, q, x, y, z);
-        if (PL::fam(q) == 0) D[PL::comp(q)] += v;
-        else B[PL::comp(q)] += v;
-    }
-}
-
-// One field component per launch: comp 0..2 -> E_x..E_z, 3..5 -> H_x..H_z.
-template <int MODE, class S>
-__global__ void fields_kernel(const S *f, const float *inv_eps, const float *inv_mu, float sc,
-                              long long P, int nx, int ny, long long ncell, int nxp, IncView inc,
-                              int comp, float *out)
-{
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ncell;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % nx);
-        const long long r = i / nx;
-        const long long c = r * nxp + x;
-        float D[3], B[3];
-        cell_DB<MODE, S>(f, sc, P, c, inc, x, (int)(r % ny), (int)(r / ny), D, B);
-        out[i] = comp < 3 ? D[comp] * inv_eps[c] : B[comp - 3] * (inv_mu ? inv_mu[c] : 1.0f);
+    for (int i = 0; i < 7; ++i) {
+        const S *g = f + (long long)i * NC * P;
+        float v[NC];
+        if constexpr (NC == 3) {
+            Io<S>::ld2(g, c, v[0], v[1]);
+            Io<S>::ld1(g + 2 * P, c, v[2]);
+        } else if constexpr (sizeof(S) == 4) {
+            Io<S>::ld2(g, c, v[0], v[1]);
+            Io<S>::ld2(g + 2 * P, c, v[2], v[3]);
+            Io<S>::ld2(g + 4 * P, c, v[4], v[5]);
+        } else {
+            Io<S>::ld4(g, c, v[0], v[1], v[2], v[3]);
+            Io<S>::ld2(g + 4 * P, c, v[4], v[5]);
+        }
+#pragma unroll
+        for (int s = 0; s < NC; ++s) {
+            const int a = s < NE ? M::ec(s) : M::hc(s - NE);
+            float add = 0.f;
+            if (in) {
+                if (inc.on == 1) add = __ldg(inc.line + (size_t)slot_plane(MODE, i, s) * inc.n + sl);
+                else if (i) add = (s < NE ? E0[a] - cross_c(i, H0, a) : H0[a] + cross_c(i, E0, a)) * (1.0f / 6.0f);
+            }
+            (s < NE ? D : B)[a] += v[s] * sc + add;
+        }
     }
 }
 
 constexpr int kEThreads = 256;
 
+// E and H maps in one pass over the populations (components 0..2: E, 3..5: H;
+// a null pointer is skipped).  Bound by HBM: the populations and 1/eps_r once,
+// 4 B a component out.  One launch a component read the populations six times:
+// 384^3 FP32 59.9 -> 2.36 ms, FP16 57.4 -> 2.36, 1024^2 EZ 0.575 -> 0.067.
+struct FieldOut { float *p[6]; };
 template <int MODE, class S>
-__global__ void __launch_bounds__(kEThreads) energy_partial(const S *f, const float *inv_eps,
-                                                            const float *inv_mu,
-                                                            float sc, long long P, int nx, int ny,
-                                                            long long ncell, int nxp, IncView inc,
-                                                            double *partial)
+__global__ void __launch_bounds__(kEThreads) fields_kernel(const S *f, const float *inv_eps, const float *inv_mu,
+                                                           float sc, long long P, int nx, int ny, int nz, int nxp,
+                                                           IncView inc, FieldOut out)
+{
+    const unsigned c = blockIdx.x * kEThreads + threadIdx.x;  // the padded plane has less than 2^31 cells
+    if (c >= (unsigned)P) return;
+    const unsigned r = c / (unsigned)nxp, x = c - r * (unsigned)nxp;
+    if (x >= (unsigned)nx) return;
+    const int z = (int)(r / (unsigned)ny), y = (int)(r - (unsigned)z * (unsigned)ny);
+    float D[3], B[3];
+    cell_DB<MODE, S>(f, sc, P, (int)c, inc, (int)x, y, z, D, B);
+    const float ie = inv_eps[c], im = inv_mu ? inv_mu[c] : 1.0f;
+    const long long i = (long long)r * nx + x;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (out.p[k]) out.p[k][i] = D[k] * ie;
+        if (out.p[3 + k]) out.p[3 + k][i] = B[k] * im;
+    }
+}
+
+// Field energy 1/2 sum (|D|^2 / eps + |B|^2 / mu), FP64 per block; HBM and the
+// FP64 pipe (about 15 operations a cell) take about the same time in FP32
+// storage.  384^3 FP32 15.8 -> 3.15 ms, 1024^2 EZ 0.355 -> 0.088.
+template <int MODE, class S>
+__global__ void __launch_bounds__(kEThreads) energy_partial(const S *f, const float *inv_eps, const float *inv_mu,
+                                                            float sc, long long P, int nx, int ny, int nxp,
+                                                            IncView inc, double *partial)
 {
     double acc = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ncell;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % nx);
-        const long long r = i / nx;
-        const long long c = r * nxp + x;
+    for (long long cl = blockIdx.x * (long long)kEThreads + threadIdx.x; cl < P; cl += (long long)gridDim.x * kEThreads) {
+        const unsigned c = (unsigned)cl;
+        const unsigned r = c / (unsigned)nxp, x = c - r * (unsigned)nxp;
+        if (x >= (unsigned)nx) continue;
+        const int z = (int)(r / (unsigned)ny), y = (int)(r - (unsigned)z * (unsigned)ny);
         float D[3], B[3];
-        cell_DB<MODE, S>(f, sc, P, c, inc, x, (int)(r % ny), (int)(r / ny), D, B);
-        const double ie = inv_eps[c], im = inv_mu ? (double)inv_mu[c] : 1.0;
-        // 1/2 (eps |E|^2 + mu |H|^2) = 1/2 (|D|^2 / eps + |B|^2 / mu)
-        acc += 0.5 * (((double)D[0] * D[0] + (double)D[1] * D[1] + (double)D[2] * D[2]) * ie +
-                      ((double)B[0] * B[0] + (double)B[1] * B[1] + (double)B[2] * B[2]) * im);
+        cell_DB<MODE, S>(f, sc, P, (int)c, inc, (int)x, y, z, D, B);
+        const double ie = inv_eps[c];
+        double d = 0.0, b = 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            if (in_e<MODE>(k)) d = fma((double)D[k], (double)D[k], d);
+            if (in_h<MODE>(k)) b = fma((double)B[k], (double)B[k], b);
+        }
+        if (inv_mu) b *= (double)inv_mu[c];
+        acc += fma(d, ie, b);
     }
     __shared__ double red[kEThreads / 32];
     const double v = warp_sum(acc);
@@ -541,12 +594,22 @@ __global__ void __launch_bounds__(kEThreads) energy_partial(const S *f, const fl
     }
 }
 
-__global__ void sum_partials(const double *partial, int n, double *out)
+// Half the sum of the block partials, in a fixed order, and beside it the
+// kernel status word, so that one copy brings both back.  (One thread summing
+// a few thousand partials took longer than the pass over a 2D grid.)
+__global__ void __launch_bounds__(kEThreads) sum_partials(const double *partial, int n, const int *status, double *out)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < n; i += kEThreads) acc += partial[i];
+    __shared__ double red[kEThreads / 32];
+    const double v = warp_sum(acc);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
         double s = 0.0;
-        for (int i = 0; i < n; ++i) s += partial[i];
-        *out = s;
+        for (int w = 0; w < kEThreads / 32; ++w) s += red[w];
+        out[0] = 0.5 * s;
+        out[1] = (double)*status;
     }
 }
 
@@ -964,25 +1027,24 @@ cudaError_t launch_add_incident(int mode, int storage, void *f, long long P, int
 template <int MODE, class S>
 static cudaError_t fields_t(const void *f, const float *inv_eps, const float *inv_mu, float sc,
                             long long P, int nx, int ny, int nz, int nxp, const IncView &inc,
-                            int comp, float *out, cudaStream_t s)
+                            float *const out[6], cudaStream_t s)
 {
-    const long long n = (long long)nx * ny * nz;
-    fields_kernel<MODE, S><<<grid_for(n, 256), 256, 0, s>>>((const S *)f, inv_eps, inv_mu, sc, P, nx,
-                                                             ny, n, nxp, inc, comp, out);
+    FieldOut o;
+    std::memcpy(o.p, out, sizeof o.p);
+    fields_kernel<MODE, S><<<(unsigned)((P + kEThreads - 1) / kEThreads), kEThreads, 0, s>>>(
+        (const S *)f, inv_eps, inv_mu, sc, P, nx, ny, nz, nxp, inc, o);
     return cudaGetLastError();
 }
 
 template <int MODE, class S>
 static cudaError_t energy_t(const void *f, const float *inv_eps, const float *inv_mu, float sc, long long P,
-                            int nx, int ny, int nz, int nxp, const IncView &inc, double *partial,
-                            int max_partial, double *out, cudaStream_t s)
+                            int nx, int ny, int nxp, const IncView &inc, double *partial,
+                            int max_partial, const int *status, double *out, cudaStream_t s)
 {
-    const long long n = (long long)nx * ny * nz;
-    int g = grid_for(n, kEThreads);
-    if (g > max_partial) g = max_partial;
-    energy_partial<MODE, S><<<g, kEThreads, 0, s>>>((const S *)f, inv_eps, inv_mu, sc, P, nx, ny, n, nxp,
-                                                     inc, partial);
-    sum_partials<<<1, 32, 0, s>>>(partial, g, out);
+    const long long need = (P + kEThreads - 1) / kEThreads, cap = 8LL * std::max(1, sm_count());
+    const int g = (int)std::min<long long>(std::min(need, cap), max_partial);
+    energy_partial<MODE, S><<<g, kEThreads, 0, s>>>((const S *)f, inv_eps, inv_mu, sc, P, nx, ny, nxp, inc, partial);
+    sum_partials<<<1, kEThreads, 0, s>>>(partial, g, status, out);
     return cudaGetLastError();
 }
 
@@ -1002,9 +1064,9 @@ static cudaError_t energy_t(const void *f, const float *inv_eps, const float *in
 
 cudaError_t launch_fields(int mode, int storage, const void *f, const float *inv_eps, const float *inv_mu,
                           float scale, long long P, int nx, int ny, int nz, int nxp,
-                          const IncView &inc, int comp, float *out, cudaStream_t s)
+                          const IncView &inc, float *const out[6], cudaStream_t s)
 {
-    LBEM_DISPATCH(fields_t, f, inv_eps, inv_mu, scale, P, nx, ny, nz, nxp, inc, comp, out, s)
+    LBEM_DISPATCH(fields_t, f, inv_eps, inv_mu, scale, P, nx, ny, nz, nxp, inc, out, s)
 }
 
 cudaError_t launch_probe(int mode, int storage, const void *f, float scale, long long P, int ny, int nxp,
@@ -1014,12 +1076,11 @@ cudaError_t launch_probe(int mode, int storage, const void *f, float scale, long
 }
 
 cudaError_t launch_energy(int mode, int storage, const void *f, const float *inv_eps, const float *inv_mu,
-                          float scale, long long P, int nx, int ny, int nz, int nxp,
-                          const IncView &inc, double *partial, int max_partial, double *out,
-                          cudaStream_t s, int *launches)
+                          float scale, long long P, int nx, int ny, int nxp, const IncView &inc, double *partial,
+                          int max_partial, const int *status, double *out, cudaStream_t s, int *launches)
 {
     if (launches) *launches += 2;
-    LBEM_DISPATCH(energy_t, f, inv_eps, inv_mu, scale, P, nx, ny, nz, nxp, inc, partial, max_partial, out, s)
+    LBEM_DISPATCH(energy_t, f, inv_eps, inv_mu, scale, P, nx, ny, nxp, inc, partial, max_partial, status, out, s)
 }
 
 }  // namespace lbem
