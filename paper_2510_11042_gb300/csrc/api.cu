@@ -1469,17 +1469,6 @@ int32_t lbem_get_time(lbem_handle h, int64_t *t_out)
     return LBEM_OK;
 }
 
-// Chunks of the far-field projection per angle: enough blocks for the face
-// cells (4096 per chunk) and for the face columns (256 per chunk).
-static int far_field_chunks(const FaceGeom &g)
-{
-    const long long cells = g.cell_start[g.nfaces];
-    long long cols = 0;
-    for (int f = 0; f < g.nfaces; ++f) cols += g.nv[f];
-    const long long c = std::max((cells + 4095) / 4096, (cols + 255) / 256);
-    return (int)std::max<long long>(1, std::min<long long>(kMaxChunks, c));
-}
-
 // The 3D projection runs as an FP32 contraction in the workspace's ff32 region.
 static void set_far_field_f32(lbem_ctx *h, FarFieldArgs &a)
 {
@@ -1521,7 +1510,6 @@ int32_t lbem_far_field(lbem_handle h, const double *theta, const double *phi, in
         a.pol[c] = h->wave.pol[c];
     }
     centre_nodes(h, &a.center_i0, &a.center_i1);
-    a.chunks = far_field_chunks(h->faces);
     double *d_theta = h->scratch;
     double *d_phi = d_theta + kAngleBatch;
     double *d_s2 = d_phi + kAngleBatch;
@@ -1535,6 +1523,7 @@ int32_t lbem_far_field(lbem_handle h, const double *theta, const double *phi, in
         a.theta = d_theta;
         a.phi = d_phi;
         a.n_ang = nb;
+        a.chunks = far_field_chunks(h->g.mode, h->faces, nb, kMaxChunks);
         a.partial = d_part;
         a.s2 = d_s2;
         a.amp = d_amp;
@@ -1986,7 +1975,7 @@ int32_t lbem_adjoint(lbem_handle h, const double *theta, const double *phi, cons
         fa.pol[c] = h->wave.pol[c];
     }
     centre_nodes(h, &fa.center_i0, &fa.center_i1);
-    fa.chunks = far_field_chunks(h->faces);
+    fa.chunks = far_field_chunks(h->g.mode, h->faces, n_ang, kMaxChunks);
     double *d_theta = h->scratch;
     double *d_phi = d_theta + kAngleBatch;
     double *d_s2 = d_phi + kAngleBatch;

@@ -397,6 +397,8 @@ struct FarFieldArgs {
 };
 cudaError_t launch_far_field(const FarFieldArgs &a, cudaStream_t s, int *launches);
 cudaError_t launch_far_field_partial(const FarFieldArgs &a, cudaStream_t s);
+// Chunks (blocks) per angle of the FP64 projection, at most `most`.
+int far_field_chunks(int mode, const FaceGeom &g, int n_ang, int most);
 
 cudaError_t launch_inv_eps(const float *eps, float *inv_eps, int nx, int ny, int nz, int nxp,
                            int *bad_flag, cudaStream_t s);

@@ -24,7 +24,7 @@ using namespace lbem;
 
 namespace {
 
-constexpr int kNoAllocChunks = 16;            // face-cell chunks per angle
+constexpr int kNoAllocChunks = 16;            // face-column chunks per angle, at most
 
 // Partial sums [angle][chunk][12]: 1024 x 16 x 12 doubles = 1.5 MB per device.
 __device__ __align__(256) double g_far_field_scratch[LBEM_NOALLOC_MAX_ANGLES * kNoAllocChunks * 12];
@@ -184,7 +184,7 @@ extern "C" int32_t lbem_far_field_noalloc(const lbem_ntff_desc *d, const double 
     a.phi = phi_dev;
     a.k = 2.0 * M_PI / d->wavelength;
     for (int c = 0; c < 3; ++c) a.center[c] = d->center[c];
-    a.chunks = kNoAllocChunks;
+    a.chunks = far_field_chunks(a.mode, a.g, n, kNoAllocChunks);
     a.partial = scratch;  // every slot is written before it is read: nothing to clear
     a.s2 = s2_dev;
     a.amp = amp_dev;

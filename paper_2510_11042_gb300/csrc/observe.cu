@@ -34,53 +34,42 @@ __device__ __forceinline__ double warp_sum(double v)
 }
 
 // ------------------------------------------------------------ far field
-// Stage 1: one block per (chunk, angle) sums w J e^{j phi}, w M e^{j phi} over
-// its share of the face cells; writes 12 doubles (Re/Im of N_xyz, L_xyz).
-// acc += w e^{j phi} (J, M) of one face cell with outward normal sgn * e_AX,
-// J = n x H, M = -n x E; (e_AX x V)_b1 = -V_b2, (e_AX x V)_b2 = V_b1.
-template <int MODE, int AX>
-__device__ __forceinline__ void face_cell(const double *base, long long plane, double sgn, double wc,
-                                          double ws, double acc[12])
+constexpr int kFFThreads = 256;
+constexpr int kFFFine = 64;         // coordinates per coarse phase entry
+constexpr int kFFTableMax = 4480;   // phase entries held in shared memory (70 KB)
+
+// How a block of far_field_columns gets its phases exp(j k r_a (p_a - c_a)):
+// evaluated at each use; as products of a coarse entry (every 64th coordinate)
+// and a fine one (the 64 offsets), tabulated per block; or from a table of
+// every coordinate of the box, filled with those products.
+enum FFPhase { FF_DIRECT = 0, FF_FACTORED = 1, FF_TABLE = 2 };
+
+__host__ __device__ inline int ff_coarse(int n) { return (n + kFFFine - 1) / kFFFine; }
+inline int ff_factored_entries(const FaceGeom &g)
 {
-    constexpr int b1 = (AX + 1) % 3, b2 = (AX + 2) % 3;
-    auto ld = [&](int slot, double &re, double &im) {
-        if (slot < 0) { re = 0.0; im = 0.0; }
-        else { re = base[(2 * slot) * plane]; im = base[(2 * slot + 1) * plane]; }
-    };
-    double Hr1, Hi1, Hr2, Hi2, Er1, Ei1, Er2, Ei2;
-    ld(slot_H(MODE, b1), Hr1, Hi1);
-    ld(slot_H(MODE, b2), Hr2, Hi2);
-    ld(slot_E(MODE, b1), Er1, Ei1);
-    ld(slot_E(MODE, b2), Er2, Ei2);
-    // J_b1 = -sgn H_b2, J_b2 = sgn H_b1, M_b1 = sgn E_b2, M_b2 = -sgn E_b1
-    const double J1r = -sgn * Hr2, J1i = -sgn * Hi2, J2r = sgn * Hr1, J2i = sgn * Hi1;
-    const double M1r = sgn * Er2, M1i = sgn * Ei2, M2r = -sgn * Er1, M2i = -sgn * Ei1;
-    acc[2 * b1 + 0] += J1r * wc - J1i * ws;
-    acc[2 * b1 + 1] += J1r * ws + J1i * wc;
-    acc[2 * b2 + 0] += J2r * wc - J2i * ws;
-    acc[2 * b2 + 1] += J2r * ws + J2i * wc;
-    acc[6 + 2 * b1 + 0] += M1r * wc - M1i * ws;
-    acc[6 + 2 * b1 + 1] += M1r * ws + M1i * wc;
-    acc[6 + 2 * b2 + 0] += M2r * wc - M2i * ws;
-    acc[6 + 2 * b2 + 1] += M2r * ws + M2i * wc;
+    int e = 0;
+    for (int ax = 0; ax < 3; ++ax) e += kFFFine + ff_coarse(g.hi[ax] - g.lo[ax] + 1);
+    return e;
 }
 
-constexpr int kFFThreads = 256;
-constexpr int kFFTableMax = 4096;   // phase-table entries held in shared memory (64 KB)
-
-// The far-field phase factorises over the coordinates of a face cell,
-//   exp(j k r.(p - c)) = prod_a exp(j k r_a (p_a - c_a)),
-// so with TABLES each block (one angle) first tabulates exp(j k r_a (p_a - c_a))
-// for every coordinate of the NTFF box along the three axes in shared memory,
-// and each (cell, angle) pair then costs two complex products instead of an
-// FP64 sincos.  Without TABLES (very large boxes) the phase is evaluated
-// directly.
-template <int MODE, bool TABLES>
-__global__ void __launch_bounds__(kFFThreads) far_field_partial(const FarFieldArgs a)
+// Stage 1: one block per (chunk of face columns, angle); writes 12 doubles
+// (Re/Im of N_xyz, L_xyz).  The phase of face cell (iu, iv) factorises as
+// t_u(iu) t_v(iv) t_w, and so does the trapezoidal weight, so one thread takes
+// one face column (fixed iv; the threads of a warp read consecutive iv,
+// coalesced) and sums the tangential phasors down the column with t_u(iu) w(iu)
+// alone; the column factor t_v(iv) w(iv) t_w multiplies the four column sums
+// once, and J = n x H, M = -n x E are formed from them.  Per (cell, angle) this
+// is four complex multiply-adds.  Bound by the FP64 pipe (two operations a
+// clock per SM), so what counts in 2D, where a column is one cell, is the
+// number of FP64 sincos: a table of every coordinate per block cost 16 blocks x
+// 1970 of them an angle on a 1024^2 grid (0.60 ms for 181 angles); factored and
+// with few blocks an angle the call takes 0.133 ms.  A 4000^2 box, too long
+// for that table, evaluated the phase of every (cell, angle): 0.97 -> 0.228 ms.
+template <int MODE, int PH>
+__global__ void __launch_bounds__(kFFThreads) far_field_columns(const FarFieldArgs a)
 {
-    extern __shared__ double tab[];  // [2 * (n0 + n1 + n2)] (re, im)
+    extern __shared__ double2 ff_tab[];
     const int ang = blockIdx.y;
-    const int chunk = blockIdx.x;
     const double th = a.theta[ang];
     double rh[3];
     if (MODE == 2) {
@@ -93,124 +82,40 @@ __global__ void __launch_bounds__(kFFThreads) far_field_partial(const FarFieldAr
         rh[1] = sin(th);
         rh[2] = 0.0;
     }
-    int toff[3];
-    if (TABLES) {
-        const int n0 = a.g.hi[0] - a.g.lo[0] + 1, n1 = a.g.hi[1] - a.g.lo[1] + 1,
-                  n2 = a.g.hi[2] - a.g.lo[2] + 1;
-        toff[0] = 0;
-        toff[1] = n0;
-        toff[2] = n0 + n1;
-        for (int e = threadIdx.x; e < n0 + n1 + n2; e += blockDim.x) {
-            const int ax = e < n0 ? 0 : (e < n0 + n1 ? 1 : 2);
-            const double pos = a.g.lo[ax] + (e - toff[ax]);
+    const int n3[3] = {a.g.hi[0] - a.g.lo[0] + 1, a.g.hi[1] - a.g.lo[1] + 1, a.g.hi[2] - a.g.lo[2] + 1};
+    // factored entries of axis ax: the 64 fine ones at foff, then the coarse ones
+    const int foff[3] = {0, kFFFine + ff_coarse(n3[0]), 2 * kFFFine + ff_coarse(n3[0]) + ff_coarse(n3[1])};
+    const int nfac = foff[2] + kFFFine + ff_coarse(n3[2]);
+    const int toff[3] = {nfac, nfac + n3[0], nfac + n3[0] + n3[1]};
+    auto cmul = [](double2 p, double2 q) { return make_double2(p.x * q.x - p.y * q.y, p.x * q.y + p.y * q.x); };
+    auto factored = [&](int ax, int e) {
+        return cmul(ff_tab[foff[ax] + kFFFine + e / kFFFine], ff_tab[foff[ax] + e % kFFFine]);
+    };
+    auto phase = [&](int ax, int e) {
+        if constexpr (PH == FF_TABLE) return ff_tab[toff[ax] + e];
+        if constexpr (PH == FF_FACTORED) return factored(ax, e);
+        double sp, cp;
+        sincos(a.k * rh[ax] * (a.g.lo[ax] + e - a.center[ax]), &sp, &cp);
+        return make_double2(cp, sp);
+    };
+    if constexpr (PH != FF_DIRECT) {
+        for (int e = threadIdx.x; e < nfac; e += blockDim.x) {
+            const int ax = e < foff[1] ? 0 : (e < foff[2] ? 1 : 2);
+            const int i = e - foff[ax];
+            const double pos = i < kFFFine ? (double)i : a.g.lo[ax] + (double)(i - kFFFine) * kFFFine - a.center[ax];
             double sp, cp;
-            sincos(a.k * rh[ax] * (pos - a.center[ax]), &sp, &cp);
-            tab[2 * e] = cp;
-            tab[2 * e + 1] = sp;
+            sincos(a.k * rh[ax] * pos, &sp, &cp);
+            ff_tab[e] = make_double2(cp, sp);
         }
         __syncthreads();
     }
-    const long long total = a.g.cell_start[a.g.nfaces];
-    const long long per = (total + a.chunks - 1) / a.chunks;
-    const long long j0 = (long long)chunk * per;
-    const long long j1 = min(total, j0 + per);
-
-    double acc[12];
-#pragma unroll
-    for (int m = 0; m < 12; ++m) acc[m] = 0.0;
-
-    for (long long j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-        int f = 0;
-        while (f + 1 < a.g.nfaces && j >= a.g.cell_start[f + 1]) ++f;
-        const long long jl = j - a.g.cell_start[f];
-        const int nu = a.g.nu[f], nv = a.g.nv[f];
-        const int iu = (int)(jl / nv), iv = (int)(jl % nv);
-        const int ax = a.g.axis[f];
-        const int ua = ax == 2 ? 1 : 2, va = ax == 0 ? 1 : 0;
-        // trapezoidal weights: 1/2 on the edges of each face
-        double w = 1.0;
-        if (nu > 1 && (iu == 0 || iu == nu - 1)) w *= 0.5;
-        if (nv > 1 && (iv == 0 || iv == nv - 1)) w *= 0.5;
-        double cp, sp;
-        if (TABLES) {
-            const int iw = a.g.side[f] ? a.g.hi[ax] - a.g.lo[ax] : 0;
-            const double *tw = tab + 2 * (toff[ax] + iw);
-            const double *tu = tab + 2 * (toff[ua] + iu);
-            const double *tv = tab + 2 * (toff[va] + iv);
-            const double pr = tu[0] * tv[0] - tu[1] * tv[1];
-            const double pi = tu[0] * tv[1] + tu[1] * tv[0];
-            cp = pr * tw[0] - pi * tw[1];
-            sp = pr * tw[1] + pi * tw[0];
-        } else {
-            double pos[3];
-            pos[ax] = a.g.side[f] ? a.g.hi[ax] : a.g.lo[ax];
-            pos[ua] = a.g.lo[ua] + iu;
-            pos[va] = a.g.lo[va] + iv;
-            const double phase = a.k * (rh[0] * (pos[0] - a.center[0]) + rh[1] * (pos[1] - a.center[1]) +
-                                        rh[2] * (pos[2] - a.center[2]));
-            sincos(phase, &sp, &cp);
+    if constexpr (PH == FF_TABLE) {
+        for (int e = threadIdx.x; e < n3[0] + n3[1] + n3[2]; e += blockDim.x) {
+            const int ax = e < n3[0] ? 0 : (e < n3[0] + n3[1] ? 1 : 2);
+            ff_tab[nfac + e] = factored(ax, e - (toff[ax] - nfac));
         }
-        const double *base = a.dft + a.g.off[f] + jl;
-        const long long plane = (long long)nu * nv;
-        const double sgn = a.g.side[f] ? 1.0 : -1.0;
-        const double wc = w * cp, ws = w * sp;
-        if (ax == 0) face_cell<MODE, 0>(base, plane, sgn, wc, ws, acc);
-        else if (ax == 1) face_cell<MODE, 1>(base, plane, sgn, wc, ws, acc);
-        else face_cell<MODE, 2>(base, plane, sgn, wc, ws, acc);
+        __syncthreads();
     }
-
-    __shared__ double red[kFFThreads / 32][12];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int m = 0; m < 12; ++m) {
-        const double v = warp_sum(acc[m]);
-        if (lane == 0) red[wid][m] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 12) {
-        double s = 0.0;
-        for (int wi = 0; wi < kFFThreads / 32; ++wi) s += red[wi][threadIdx.x];
-        a.partial[((long long)ang * a.chunks + chunk) * 12 + threadIdx.x] = s;
-    }
-}
-
-// Column form of stage 1 (phase tables in shared memory).  The phase of face
-// cell (iu, iv) factorises as t_u(iu) t_v(iv) t_w, and so does the
-// trapezoidal weight, so one thread takes one face column (fixed iv; the
-// threads of a warp read consecutive iv, coalesced) and sums the tangential
-// phasors down the column with t_u(iu) w(iu) alone; the column factor
-// t_v(iv) w(iv) t_w multiplies the four column sums once, and J = n x H,
-// M = -n x E are formed from them.  Per (cell, angle) this is four complex
-// multiply-adds.  Blocks stride over chunks of kFFThreads columns.
-template <int MODE>
-__global__ void __launch_bounds__(kFFThreads) far_field_columns(const FarFieldArgs a)
-{
-    extern __shared__ double tab[];  // [2 * (n0 + n1 + n2)] (re, im)
-    const int ang = blockIdx.y;
-    const double th = a.theta[ang];
-    double rh[3];
-    if (MODE == 2) {
-        const double ph = a.phi[ang];
-        rh[0] = sin(th) * cos(ph);
-        rh[1] = sin(th) * sin(ph);
-        rh[2] = cos(th);
-    } else {
-        rh[0] = cos(th);
-        rh[1] = sin(th);
-        rh[2] = 0.0;
-    }
-    const int n0 = a.g.hi[0] - a.g.lo[0] + 1, n1 = a.g.hi[1] - a.g.lo[1] + 1,
-              n2 = a.g.hi[2] - a.g.lo[2] + 1;
-    const int toff[3] = {0, n0, n0 + n1};
-    for (int e = threadIdx.x; e < n0 + n1 + n2; e += blockDim.x) {
-        const int ax = e < n0 ? 0 : (e < n0 + n1 ? 1 : 2);
-        const double pos = a.g.lo[ax] + (e - toff[ax]);
-        double sp, cp;
-        sincos(a.k * rh[ax] * (pos - a.center[ax]), &sp, &cp);
-        tab[2 * e] = cp;
-        tab[2 * e + 1] = sp;
-    }
-    __syncthreads();
 
     int ncols = 0;
     for (int f = 0; f < a.g.nfaces; ++f) ncols += a.g.nv[f];
@@ -218,65 +123,62 @@ __global__ void __launch_bounds__(kFFThreads) far_field_columns(const FarFieldAr
 #pragma unroll
     for (int m = 0; m < 12; ++m) acc[m] = 0.0;
 
-    for (int col = blockIdx.x * kFFThreads + threadIdx.x; col < ncols; col += a.chunks * kFFThreads) {
-        int f = 0, iv = col;
-        while (iv >= a.g.nv[f]) iv -= a.g.nv[f++];
+    // the columns of one face at a time, so that the components are compile-time
+    auto column = [&](auto axis, int f, int iv) {
+        constexpr int ax = decltype(axis)::value;
+        constexpr int ua = ax == 2 ? 1 : 2, va = ax == 0 ? 1 : 0;
+        constexpr int b1 = (ax + 1) % 3, b2 = (ax + 2) % 3;
+        constexpr int slot[4] = {slot_H(MODE, b1), slot_H(MODE, b2), slot_E(MODE, b1), slot_E(MODE, b2)};
         const int nu = a.g.nu[f], nv = a.g.nv[f];
-        const int ax = a.g.axis[f];
-        const int ua = ax == 2 ? 1 : 2, va = ax == 0 ? 1 : 0;
-        const int b1 = (ax + 1) % 3, b2 = (ax + 2) % 3;
-        const int sH1 = slot_H(MODE, b1), sH2 = slot_H(MODE, b2);
-        const int sE1 = slot_E(MODE, b1), sE2 = slot_E(MODE, b2);
         const long long plane = (long long)nu * nv;
         const double *base = a.dft + a.g.off[f] + iv;
-        const double *tu = tab + 2 * toff[ua];
         // column sums of t_u w_u X for X = H_b1, H_b2, E_b1, E_b2 (re, im)
-        double sH1r = 0, sH1i = 0, sH2r = 0, sH2i = 0, sE1r = 0, sE1i = 0, sE2r = 0, sE2i = 0;
-        for (int iu = 0; iu < nu; ++iu) {
-            double pr = tu[2 * iu], pi = tu[2 * iu + 1];
-            if (nu > 1 && (iu == 0 || iu == nu - 1)) {
-                pr *= 0.5;
-                pi *= 0.5;
-            }
-            const double *c = base + (long long)iu * nv;
-            if (sH1 >= 0) {
-                const double xr = c[(2 * sH1) * plane], xi = c[(2 * sH1 + 1) * plane];
-                sH1r = fma(pr, xr, fma(-pi, xi, sH1r));
-                sH1i = fma(pr, xi, fma(pi, xr, sH1i));
-            }
-            if (sH2 >= 0) {
-                const double xr = c[(2 * sH2) * plane], xi = c[(2 * sH2 + 1) * plane];
-                sH2r = fma(pr, xr, fma(-pi, xi, sH2r));
-                sH2i = fma(pr, xi, fma(pi, xr, sH2i));
-            }
-            if (sE1 >= 0) {
-                const double xr = c[(2 * sE1) * plane], xi = c[(2 * sE1 + 1) * plane];
-                sE1r = fma(pr, xr, fma(-pi, xi, sE1r));
-                sE1i = fma(pr, xi, fma(pi, xr, sE1i));
-            }
-            if (sE2 >= 0) {
-                const double xr = c[(2 * sE2) * plane], xi = c[(2 * sE2 + 1) * plane];
-                sE2r = fma(pr, xr, fma(-pi, xi, sE2r));
-                sE2i = fma(pr, xi, fma(pi, xr, sE2i));
+        double sr[4] = {0, 0, 0, 0}, si[4] = {0, 0, 0, 0};
+        if constexpr (MODE != 2) {  // one cell a column, t_u = 1
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (slot[q] >= 0) {
+                    sr[q] = base[(2 * slot[q]) * plane];
+                    si[q] = base[(2 * slot[q] + 1) * plane];
+                }
+        } else {
+            for (int iu = 0; iu < nu; ++iu) {
+                double2 p = phase(ua, iu);
+                if (nu > 1 && (iu == 0 || iu == nu - 1)) {
+                    p.x *= 0.5;
+                    p.y *= 0.5;
+                }
+                const double *c = base + (long long)iu * nv;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const double xr = c[(2 * slot[q]) * plane], xi = c[(2 * slot[q] + 1) * plane];
+                    sr[q] = fma(p.x, xr, fma(-p.y, xi, sr[q]));
+                    si[q] = fma(p.x, xi, fma(p.y, xr, si[q]));
+                }
             }
         }
         // column factor t_v(iv) w_v(iv) t_w and the outward normal's sign
-        const int iw = a.g.side[f] ? a.g.hi[ax] - a.g.lo[ax] : 0;
-        const double *tv = tab + 2 * (toff[va] + iv), *tw = tab + 2 * (toff[ax] + iw);
-        double wv = 1.0;
-        if (nv > 1 && (iv == 0 || iv == nv - 1)) wv = 0.5;
-        const double sgn = a.g.side[f] ? 1.0 : -1.0;
-        const double cr = wv * (tv[0] * tw[0] - tv[1] * tw[1]);
-        const double ci = wv * (tv[0] * tw[1] + tv[1] * tw[0]);
+        double2 cf = cmul(phase(va, iv), phase(ax, a.g.side[f] ? n3[ax] - 1 : 0));
+        const double w = (nv > 1 && (iv == 0 || iv == nv - 1) ? 0.5 : 1.0) * (a.g.side[f] ? 1.0 : -1.0);
+        cf.x *= w;
+        cf.y *= w;
         // J_b1 = -sgn H_b2, J_b2 = sgn H_b1, M_b1 = sgn E_b2, M_b2 = -sgn E_b1
         auto add = [&](int m, double s, double xr, double xi) {
-            acc[m] += s * (cr * xr - ci * xi);
-            acc[m + 1] += s * (cr * xi + ci * xr);
+            acc[m] = fma(s * cf.x, xr, fma(-s * cf.y, xi, acc[m]));
+            acc[m + 1] = fma(s * cf.x, xi, fma(s * cf.y, xr, acc[m + 1]));
         };
-        add(2 * b1, -sgn, sH2r, sH2i);
-        add(2 * b2, sgn, sH1r, sH1i);
-        add(6 + 2 * b1, sgn, sE2r, sE2i);
-        add(6 + 2 * b2, -sgn, sE1r, sE1i);
+        if (slot[1] >= 0) add(2 * b1, -1.0, sr[1], si[1]);
+        if (slot[0] >= 0) add(2 * b2, 1.0, sr[0], si[0]);
+        if (slot[3] >= 0) add(6 + 2 * b1, 1.0, sr[3], si[3]);
+        if (slot[2] >= 0) add(6 + 2 * b2, -1.0, sr[2], si[2]);
+    };
+    for (int col = blockIdx.x * kFFThreads + threadIdx.x; col < ncols; col += a.chunks * kFFThreads) {
+        int f = 0, iv = col;
+        while (iv >= a.g.nv[f]) iv -= a.g.nv[f++];
+        const int ax = a.g.axis[f];
+        if (ax == 0) column(std::integral_constant<int, 0>(), f, iv);
+        else if (ax == 1) column(std::integral_constant<int, 1>(), f, iv);
+        else if (MODE == 2) column(std::integral_constant<int, 2>(), f, iv);
     }
 
     __shared__ double red[kFFThreads / 32][12];
@@ -825,17 +727,6 @@ __global__ void __launch_bounds__(kF32Threads, 2) far_field_f32(const FarFieldAr
 
 }  // namespace
 
-#define LBEM_FF_TABLES(MODE)                                                                 \
-    do {                                                                                     \
-        if (smem > 48 * 1024) {                                                              \
-            cudaError_t e_ = cudaFuncSetAttribute(far_field_columns<MODE>,                   \
-                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                                  kFFTableMax * 2 * (int)sizeof(double));    \
-            if (e_ != cudaSuccess) return e_;                                                \
-        }                                                                                    \
-        far_field_columns<MODE><<<g1, kFFThreads, smem, s>>>(a);                             \
-    } while (0)
-
 static size_t ff32_smem(int uc)
 {
     return (size_t)uc * kF32Angles * sizeof(float2) + (size_t)kF32Rows * 4 * 32 * sizeof(float4) +
@@ -917,43 +808,66 @@ static cudaError_t launch_far_field_f32(FarFieldArgs a, cudaStream_t s, int *lau
     return cudaGetLastError();
 }
 
-cudaError_t launch_far_field(const FarFieldArgs &a, cudaStream_t s, int *launches)
+// The FP64 projection's partial sums (the caller finalises).  In 3D a column
+// has many cells, so every coordinate's phase is tabulated where that fits; 2D
+// boxes use each entry once and take the factored phases.
+template <int MODE, int PH>
+static cudaError_t far_field_columns_go(const FarFieldArgs &a, int entries, cudaStream_t s)
 {
-    if (a.mode == 2 && a.x32 != nullptr) return launch_far_field_f32(a, s, launches);
-    dim3 g1(a.chunks, a.n_ang);
-    const int entries = (a.g.hi[0] - a.g.lo[0] + 1) + (a.g.hi[1] - a.g.lo[1] + 1) + (a.g.hi[2] - a.g.lo[2] + 1);
-    const bool tables = entries <= kFFTableMax;
-    const size_t smem = tables ? (size_t)entries * 2 * sizeof(double) : 0;
-    switch (a.mode * 2 + (tables ? 1 : 0)) {
-    case 0: far_field_partial<0, false><<<g1, kFFThreads, 0, s>>>(a); break;
-    case 1: LBEM_FF_TABLES(0); break;
-    case 2: far_field_partial<1, false><<<g1, kFFThreads, 0, s>>>(a); break;
-    case 3: LBEM_FF_TABLES(1); break;
-    case 4: far_field_partial<2, false><<<g1, kFFThreads, 0, s>>>(a); break;
-    case 5: LBEM_FF_TABLES(2); break;
-    default: return cudaErrorInvalidValue;
+    const size_t smem = (size_t)entries * sizeof(double2);
+    if (smem > 47 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(far_field_columns<MODE, PH>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   kFFTableMax * (int)sizeof(double2));
+        if (e != cudaSuccess) return e;
     }
-    far_field_finalize<<<(a.n_ang + 127) / 128, 128, 0, s>>>(a);
-    if (launches) *launches += 2;
+    far_field_columns<MODE, PH><<<dim3(a.chunks, a.n_ang), kFFThreads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
-// The projection's partial-sum stage alone (the caller finalises).
+template <int MODE>
+static cudaError_t far_field_columns_t(const FarFieldArgs &a, cudaStream_t s)
+{
+    const int fac = ff_factored_entries(a.g);
+    if constexpr (MODE == 2) {
+        int all = fac;
+        for (int ax = 0; ax < 3; ++ax) all += a.g.hi[ax] - a.g.lo[ax] + 1;
+        if (all <= kFFTableMax) return far_field_columns_go<MODE, FF_TABLE>(a, all, s);
+    }
+    if (fac <= kFFTableMax) return far_field_columns_go<MODE, FF_FACTORED>(a, fac, s);
+    return far_field_columns_go<MODE, FF_DIRECT>(a, 0, s);
+}
+
 cudaError_t launch_far_field_partial(const FarFieldArgs &a, cudaStream_t s)
 {
-    dim3 g1(a.chunks, a.n_ang);
-    const int entries = (a.g.hi[0] - a.g.lo[0] + 1) + (a.g.hi[1] - a.g.lo[1] + 1) + (a.g.hi[2] - a.g.lo[2] + 1);
-    const bool tables = entries <= kFFTableMax;
-    const size_t smem = tables ? (size_t)entries * 2 * sizeof(double) : 0;
-    switch (a.mode * 2 + (tables ? 1 : 0)) {
-    case 0: far_field_partial<0, false><<<g1, kFFThreads, 0, s>>>(a); break;
-    case 1: LBEM_FF_TABLES(0); break;
-    case 2: far_field_partial<1, false><<<g1, kFFThreads, 0, s>>>(a); break;
-    case 3: LBEM_FF_TABLES(1); break;
-    case 4: far_field_partial<2, false><<<g1, kFFThreads, 0, s>>>(a); break;
-    case 5: LBEM_FF_TABLES(2); break;
+    switch (a.mode) {
+    case 0: return far_field_columns_t<0>(a, s);
+    case 1: return far_field_columns_t<1>(a, s);
+    case 2: return far_field_columns_t<2>(a, s);
     default: return cudaErrorInvalidValue;
     }
+}
+
+// Blocks an angle of the FP64 projection: in 2D about three blocks per SM in
+// all (each block pays for its phase entries), in 3D one per 4096 face cells;
+// at most one per kFFThreads columns.
+int far_field_chunks(int mode, const FaceGeom &g, int n_ang, int most)
+{
+    long long cols = 0;
+    for (int f = 0; f < g.nfaces; ++f) cols += g.nv[f];
+    const long long per_cols = (cols + kFFThreads - 1) / kFFThreads;
+    long long c = std::max((g.cell_start[g.nfaces] + 4095) / 4096, per_cols);
+    if (mode != 2) c = std::min<long long>(per_cols, (3LL * std::max(1, sm_count()) + n_ang - 1) / std::max(1, n_ang));
+    return (int)std::max<long long>(1, std::min<long long>(most, c));
+}
+
+cudaError_t launch_far_field(const FarFieldArgs &a, cudaStream_t s, int *launches)
+{
+    if (a.mode == 2 && a.x32 != nullptr) return launch_far_field_f32(a, s, launches);
+    const cudaError_t e = launch_far_field_partial(a, s);
+    if (e != cudaSuccess) return e;
+    far_field_finalize<<<(a.n_ang + 127) / 128, 128, 0, s>>>(a);
+    if (launches) *launches += 2;
     return cudaGetLastError();
 }
 
