@@ -67,6 +67,14 @@ struct lbem_ctx {
     bool xs_wide = false;       // a step staged faces beyond x that the step stream has not summed
     unsigned xs_masks[kXBank];
     double xs_sc[kXBank], xs_ss[kXBank];
+    // 2D passes of kMarchSteps steps (march.cu): moments of the incident line
+    // at 2 kMarchSteps times (time t at t mod that), and the time up to which
+    // they and line(line_front) are valid (-1: none); staged face fields
+    float *lm = nullptr;
+    int64_t line_front = -1;
+    int ms_cap = 0, ms_cnt = 0;  // staging slots, and those filled
+    long long ms_n = 0;          // cells of all faces
+    double ms_sc[kMarchStage], ms_ss[kMarchStage];
     cudaStream_t fstream = nullptr;           // side stream of the bank sums (3D)
     cudaEvent_t xs_filled[2] = {nullptr, nullptr};
     cudaEvent_t xs_summed[2] = {nullptr, nullptr};
@@ -166,6 +174,8 @@ struct Layout {
     size_t f0, f1, inv_eps, inv_mu, pw_tab, line[kLineBufs], dft, line_dft, scratch, ff32, stage, flag, total;
     size_t x32_cap, tab32_cap;  // float2 capacities of the 3D FP32 far field (0 in 2D)
     size_t xstage, xstage_floats;  // staged face DFT fields
+    size_t lm;                     // 2D: moments of the incident line
+    int ms_cap;                    // 2D: staging slots
     size_t aa_faces;               // in-place streaming: FI and FO of the six directions
     long long fplane[3];           // face cells of each axis (0 along 1-cell axes)
     int Q, nxp, n_line_max;
@@ -251,7 +261,15 @@ static Layout make_layout(const lbem_grid_desc *g)
     L.xstage_floats = g->mode == 2 ? (size_t)kXStage * NC * 2 *
                                          ((size_t)g->ny * g->nz + (size_t)g->nx * g->nz + (size_t)g->nx * g->ny)
                                    : 0;
+    // 2D: up to kMarchStage steps of the four faces (64 MB at most, but one pass)
+    L.ms_cap = 0;
+    if (g->mode != 2) {
+        const long long faces = 2LL * ((long long)g->nx + g->ny), fit = (16LL << 20) / (3 * faces);
+        L.ms_cap = (int)std::max<long long>(1, std::min<long long>(kMarchStage, fit) / kMarchSteps) * kMarchSteps;
+        L.xstage_floats = (size_t)L.ms_cap * 3 * faces;
+    }
     L.xstage = take(L.xstage_floats * 4);
+    L.lm = take(g->mode != 2 ? (size_t)2 * kMarchSteps * NC * L.n_line_max * 4 : 0);
     L.stage = take((size_t)L.ncell * 4);
     L.flag = take(256);
     L.total = o;
@@ -480,6 +498,8 @@ int32_t lbem_create(const lbem_grid_desc *grid, int32_t velocity_set, const floa
     h->scratch_doubles = L.scratch_doubles;
     h->xstage = (float *)(h->ws + L.xstage);
     h->xstage_floats = L.xstage_floats;
+    h->lm = (float *)(h->ws + L.lm);
+    h->ms_cap = L.ms_cap;
     h->x32_cap = L.x32_cap;
     h->tab32_cap = L.tab32_cap;
     h->x32 = L.x32_cap ? (float2 *)(h->ws + L.ff32) : nullptr;
@@ -577,6 +597,9 @@ static void build_faces(lbem_ctx *h)
     h->xs_bank = 0;
     h->xs_cnt = 0;
     h->xs_wide = false;
+    // 2D: the four faces of a box in x and y
+    h->ms_n = (h->g.mode != 2 && F.nfaces == 4) ? cells : 0;
+    h->ms_cnt = 0;
 }
 
 static int inject_analytic(lbem_ctx *h, const lbem_plane_wave *w);
@@ -633,6 +656,7 @@ int32_t lbem_inject_plane_wave(lbem_handle h, const lbem_plane_wave *w)
         CK(h, cudaStreamSynchronize(h->stream));
     }
     h->adj_valid = false;
+    h->line_front = -1;
     h->wave = *w;
     h->wave.source_index = src;
     h->has_wave = true;
@@ -751,6 +775,7 @@ static int inject_analytic(lbem_ctx *h, const lbem_plane_wave *w)
     } else {
         h->faces.nfaces = 0;
         h->xs_n = 0;
+        h->ms_n = 0;
         h->faces.cell_start[0] = 0;
         h->dft_doubles = 0;
     }
@@ -926,12 +951,156 @@ static void aa_aim(lbem_ctx *h, StepArgs &a, int kind)
 // closed-form source.
 static int step_variant(const lbem_ctx *h) { return h->analytic ? 2 : (h->mu_on ? 1 : 0); }
 
-// Whether lbem_step takes two steps per pass: fusion on, on a grid whose
-// blocks fill the GPU.
+// Whether lbem_step takes several steps per pass: fusion on, and in 3D two on
+// a grid whose blocks fill the GPU, in 2D kMarchSteps on any grid.
 static bool two_step_passes(lbem_ctx *h)
 {
-    return h->fuse == 2 && !h->aa &&
-           step2_worthwhile(h->g.mode, h->g.storage, step_variant(h), h->g.nx, h->g.ny, h->g.nz, h->share);
+    return h->fuse == 2 && !h->aa && h->g.mode == 2 &&
+           step2_worthwhile(h->g.storage, step_variant(h), h->g.nx, h->g.ny, h->g.nz);
+}
+
+static bool march_passes(const lbem_ctx *h)
+{
+    return h->fuse == 2 && !h->aa && !h->analytic && march_fits(h->g.mode, h->g.nx, h->g.ny, h->g.nz);
+}
+
+// Sum the staged 2D face fields into the DFT accumulators on the step stream.
+static int flush_march(lbem_ctx *h)
+{
+    if (h->ms_cnt == 0) return LBEM_OK;
+    DftFlush2dArgs f;
+    f.stage = h->xstage;
+    f.n = h->ms_n;
+    f.cnt = h->ms_cnt;
+    f.dft = h->dft;
+    for (int k = 0; k < 4; ++k) {
+        f.start[k] = h->faces.cell_start[k];
+        f.plane[k] = (long long)h->faces.nu[k] * h->faces.nv[k];
+        f.face_off[k] = h->faces.off[k];
+    }
+    f.start[4] = h->faces.cell_start[4];
+    std::memcpy(f.sc, h->ms_sc, sizeof f.sc);
+    std::memcpy(f.ss, h->ms_ss, sizeof f.ss);
+    h->ms_cnt = 0;
+    CK(h, launch_dft_flush_2d(f, h->stream));
+    h->launches += 1;
+    return LBEM_OK;
+}
+
+static float *lm_at(lbem_ctx *h, int64_t t)
+{
+    return h->lm + (size_t)(t % (2 * kMarchSteps)) * h->NC * h->n_line_max;
+}
+
+// What does not change between a run's passes.
+static void march_common(lbem_ctx *h, MarchArgs &m)
+{
+    std::memset(&m, 0, sizeof m);
+    m.inv_eps = h->inv_eps;
+    m.inv_mu = h->mu_on ? h->inv_mu : nullptr;
+    m.status = h->flag + 1;
+    m.nx = h->g.nx; m.ny = h->g.ny; m.nxp = h->nxp;
+    m.P = h->P;
+    m.w = h->g.absorber_width;
+    m.sigma_max = (float)h->g.sigma_max;
+    m.inv_w = m.w > 0 ? 1.0f / (float)m.w : 0.f;
+    m.scale = h->scale;
+    m.inv_scale = h->inv_scale;
+    for (int k = 0; k < 2; ++k) m.nt_lo[k] = m.nt_hi[k] = -8;
+    if (!h->has_wave) return;
+    m.tfsf = 1;
+    for (int k = 0; k < 2; ++k) {
+        m.tf_lo[k] = h->wave.tfsf_lo[k];
+        m.tf_hi[k] = h->wave.tfsf_hi[k];
+        m.nt_lo[k] = h->wave.ntff_lo[k];
+        m.nt_hi[k] = h->wave.ntff_hi[k];
+    }
+    m.inc_axis = h->inc_axis;
+    m.n_line = h->n_line;
+    m.xs_n = h->ms_n;
+    if (h->ms_n)
+        for (int k = 0; k < 4; ++k) m.xs_start[k] = h->faces.cell_start[k];
+    LineMarch &l = m.line;
+    l.n = h->n_line;
+    l.axis = h->inc_axis;
+    l.w = m.w;
+    l.sigma_max = m.sigma_max;
+    l.inv_w = m.inv_w;
+    l.src_index = h->src_index;
+    l.dft = h->line_dft;
+}
+
+static void march_buffers(MarchArgs &m, const void *in, void *out, size_t plane_bytes)
+{
+    for (int i = 0; i < 7; ++i)
+        for (int k = 0; k < 2; ++k) {
+            m.fin[2 * i + k] = (const char *)in + (size_t)(3 * i + 2 * k) * plane_bytes;
+            m.fout[2 * i + k] = (char *)out + (size_t)(3 * i + 2 * k) * plane_bytes;
+        }
+}
+
+// kMarchSteps steps in one pass: level n from f[cur] to f[cur ^ 1].  The pass
+// needs the line's moments at its own times and advances the line for the
+// next one; where the previous pass did not (a first pass, or single steps
+// since), a small launch starts it.
+static int march_pass(lbem_ctx *h, MarchArgs &m)
+{
+    constexpr int K = kMarchSteps;
+    const int64_t n = h->t;
+    const int cnt0 = h->ms_cnt;
+    march_buffers(m, h->f[h->cur], h->f[h->cur ^ 1], (size_t)h->P * h->elem);
+    m.dft_mask = 0;
+    if (h->has_wave) {
+        LineMarch &l = m.line;
+        if (h->line_front != n + K) {
+            LineMarch st = l;
+            st.dft_mask = 0;
+            st.from = line_at(h, n + 1);
+            st.steps = K - 1;
+            st.lm_from = lm_at(h, n + 1);
+            for (int k = 0; k < K; ++k) {
+                st.lm[k] = lm_at(h, n + 2 + k);
+                st.full[k] = k == K - 2 ? line_at(h, n + K) : nullptr;
+                source_fields(h, n + 2 + k, st.src_E[k], st.src_H[k]);
+            }
+            CK(h, launch_line_start(h->g.mode, st, h->stream));
+            h->launches += 1;
+            h->line_front = n + K;
+        }
+        l.from = line_at(h, n + K);
+        l.steps = K;
+        l.dft_mask = 0;
+        for (int k = 0; k < K; ++k) {
+            const int64_t t = n + 1 + k, tl = n + K + 1 + k;
+            m.lm[k] = l.lm_now[k] = lm_at(h, t);
+            l.lm[k] = lm_at(h, tl);
+            l.full[k] = (k == 0 || k == K - 1) ? line_at(h, tl) : nullptr;
+            source_fields(h, tl, l.src_E[k], l.src_H[k]);
+            if (h->ms_n == 0 || h->dft_t0 < 1 || t < h->dft_t0 || t >= h->dft_t0 + (int64_t)h->dft_periods * h->T)
+                continue;
+            const double ph = 2.0 * M_PI * (double)(t % h->T) / (double)h->T;
+            const double c = std::cos(ph), s = std::sin(ph), sc = 2.0 / ((double)h->dft_periods * h->T);
+            m.dft_mask |= 1u << k;
+            l.dft_mask |= 1u << k;
+            l.dft_scale = sc;
+            l.dft_c[k] = c;
+            l.dft_s[k] = s;
+            m.stage[k] = h->xstage + (size_t)h->ms_cnt * 3 * h->ms_n;
+            h->ms_sc[h->ms_cnt] = sc * h->scale * c;
+            h->ms_ss[h->ms_cnt] = sc * h->scale * s;
+            ++h->ms_cnt;
+        }
+    }
+    const cudaError_t e = launch_march(h->g.mode, h->g.storage, m, false, h->share, h->stream);
+    if (e != cudaSuccess) {
+        h->ms_cnt = cnt0;
+        return cuda_fail(h, e, "2D pass launch");
+    }
+    h->launches += 1;
+    if (h->has_wave) h->line_front = n + 2 * K;
+    h->cur ^= 1;
+    h->t += K;
+    return LBEM_OK;
 }
 
 // The steps of lbem_step; on an error the step stream is still joined with
@@ -940,15 +1109,22 @@ static int step_loop(lbem_ctx *h, int64_t n)
 {
     StepArgs a;
     fill_common_args(h, a);
-    const bool pairs = two_step_passes(h);
-    StepArgs a2, la[2];
-    if (pairs) {
-        fill_common_args(h, a2);
-        fill_common_args(h, la[0]);
-        fill_common_args(h, la[1]);
-    }
-    bool line_ready = false;  // the previous pass advanced the incident line for this one
+    const bool pairs = two_step_passes(h), march = march_passes(h);
+    StepArgs a2;
+    if (pairs) fill_common_args(h, a2);
+    MarchArgs m;
+    if (march) march_common(h, m);
     for (int64_t k = 0; k < n;) {
+        if (march && n - k >= kMarchSteps) {
+            if (h->ms_cnt + kMarchSteps > h->ms_cap) {
+                const int rc = flush_march(h);
+                if (rc != LBEM_OK) return rc;
+            }
+            const int rc = march_pass(h, m);
+            if (rc != LBEM_OK) return rc;
+            k += kMarchSteps;
+            continue;
+        }
         if (pairs && n - k >= 2) {
             // two steps in one pass: level n from f[cur], level n+2 into f[cur ^ 1]
             if (h->xs_cnt + 2 > kXBank) {
@@ -960,21 +1136,12 @@ static int step_loop(lbem_ctx *h, int64_t n)
             const int cnt0 = h->xs_cnt;
             stage_slot(h, a, h->xs_allmask);
             stage_slot(h, a2, h->xs_allmask);
-            // a 2D pass that another pass of this call follows advances the
-            // incident line for it (the line work of steps t+2 and t+3)
-            const bool ahead = a.line_on && h->g.mode != 2 && n - k >= 4;
-            if (ahead) {
-                step_args_at(h, la[0], h->t + 2, h->cur, h->cur ^ 1);
-                step_args_at(h, la[1], h->t + 3, h->cur ^ 1, h->cur ^ 1);
-            }
-            cudaError_t e = launch_step2(h->g.mode, h->g.storage, step_variant(h), a, a2, h->stream, h->share,
-                                         ahead ? la : nullptr, line_ready);
+            cudaError_t e = launch_step2(h->g.storage, step_variant(h), a, a2, h->stream);
             if (e != cudaSuccess) {
                 h->xs_cnt = cnt0;   // the claimed slots hold nothing
                 return cuda_fail(h, e, "two-step kernel launch");
             }
-            h->launches += (a.line_on && !line_ready) ? 2 : 1;
-            line_ready = ahead;
+            h->launches += a.line_on ? 2 : 1;
             h->cur ^= 1;
             h->t += 2;
             k += 2;
@@ -986,7 +1153,8 @@ static int step_loop(lbem_ctx *h, int64_t n)
                 const int rc = flush_x_stage(h, false);
                 if (rc != LBEM_OK) return rc;
             }
-            line_ready = false;
+            const int rc2 = flush_march(h);
+            if (rc2 != LBEM_OK) return rc2;
             const int kind = h->aa_phase;  // in-place streaming: 0 push, 1 in place
             if (h->aa && kind == 0 && !h->aa_fi_valid) {
                 CK(h, launch_aa_fill(h->g.mode, h->g.storage, h->f[0], h->P, h->g.nx, h->g.ny, h->g.nz, h->nxp,
@@ -1026,6 +1194,8 @@ static int step_loop(lbem_ctx *h, int64_t n)
             if (rc != LBEM_OK) return rc;
         }
     }
+    const int rc = flush_march(h);
+    if (rc != LBEM_OK) return rc;
     return flush_x_stage(h, false);  // every call leaves the DFT complete on the step stream
 }
 
@@ -1054,7 +1224,7 @@ int32_t lbem_set_step_fusion(lbem_handle h, int32_t steps_per_pass)
 int32_t lbem_get_step_fusion(lbem_handle h, int32_t *steps_per_pass)
 {
     if (!h || !steps_per_pass) return fail(h, LBEM_ERR_ARG, "NULL argument");
-    *steps_per_pass = two_step_passes(h) ? 2 : 1;
+    *steps_per_pass = two_step_passes(h) || march_passes(h) ? 2 : 1;
     return LBEM_OK;
 }
 
@@ -1759,6 +1929,7 @@ int32_t lbem_load_state(lbem_handle h, const void *buf, size_t bytes)
         hd.mode != h->g.mode || hd.storage != h->g.storage || hd.Q != h->Q)
         return fail(h, LBEM_ERR_ARG, "snapshot does not match this grid");
     h->adj_valid = false;
+    h->line_front = -1;
     const char *p = (const char *)buf + sizeof hd;
     if (h->aa) {  // the snapshot replaces the whole state, in the canonical layout
         h->aa_phase = 0;

@@ -13,9 +13,9 @@
 namespace lbem {
 
 constexpr int kMaxDevices = 64;  // per-device set-up caches
-// Buffers of the incident line: a two-step pass reads line(n+1) and line(n+2)
-// while its first block may already advance the line for the next pass,
-// reading line(n+3) and writing line(n+4) and line(n+5).
+// Buffers of the incident line, line(t) in buffer t mod kLineBufs: a 2D pass
+// from time n to n + 4 reads line(n+4) and writes line(n+5) and line(n+8),
+// after which line(n+4), line(n+5) and line(n+8) are in use.
 constexpr int kLineBufs = 5;
 // Streaming multiprocessors and L2 bytes of the current device (queried once
 // per device; 0 if the query fails).
@@ -276,20 +276,14 @@ cudaError_t launch_batch(int mode, int storage, const BatchArgs &b, int grid, cu
 cudaError_t launch_barrier_selftest(const BatchArgs &b, cudaStream_t s);
 int batch_max_blocks_per_sm(int mode, int storage);
 cudaError_t launch_step(int mode, int storage, const StepArgs &a, cudaStream_t s);
-// Two steps in one pass (any mode and storage; variant 0: plain update, 1:
-// with the per-cell mu_r map; 2, the closed-form source, is refused and
-// reported not worthwhile): s1 the first
-// step's arguments (reads fin_q), s2 the second's (writes fout_q, which must
-// not alias s1.fin_q); with the incident line on, a one-block launch before
-// it updates the line for both steps (two launches in all).
-// share: how many grids step concurrently beside each other (the lanes of a
-// batched run), which the choice and the launch shape take into account.
-// ahead (2D, incident line on): the arguments of the next pass's two steps,
-// whose line work the first block does (line(n+4), line(n+5)); line_ready: the
-// previous pass did this pass's line work, so the one-block launch is left out.
-cudaError_t launch_step2(int mode, int storage, int variant, const StepArgs &s1, const StepArgs &s2,
-                         cudaStream_t s, int share = 1, const StepArgs *ahead = nullptr, bool line_ready = false);
-bool step2_worthwhile(int mode, int storage, int variant, int nx, int ny, int nz, int share = 1);
+// Two steps in one pass (3D, any storage; variant 0: plain update, 1: with the
+// per-cell mu_r map; 2, the closed-form source, is refused and reported not
+// worthwhile): s1 the first step's arguments (reads fin_q), s2 the second's
+// (writes fout_q, which must not alias s1.fin_q); with the incident line on, a
+// one-block launch before it updates the line for both steps (two launches in
+// all).
+cudaError_t launch_step2(int storage, int variant, const StepArgs &s1, const StepArgs &s2, cudaStream_t s);
+bool step2_worthwhile(int storage, int variant, int nx, int ny, int nz);
 
 // In-place streaming on one population buffer (aa.cu).  Face buffers of
 // direction i = 1..6 on axis (i - 1) / 2 ([NC][fplane[axis]] storage
@@ -324,6 +318,65 @@ cudaError_t launch_fill(float *p, long long n, float v, cudaStream_t s);
 cudaError_t launch_line_init(int mode, const StepArgs &a, cudaStream_t s);
 // The step kernel with a.rec written (FP32 storage; forward replay of the adjoint)
 cudaError_t launch_step_record(int mode, const StepArgs &a, cudaStream_t s);
+
+// ---- four steps per pass in 2D (march.cu)
+constexpr int kMarchSteps = 4;
+constexpr int kMarchStage = 64;    // staged steps of NTFF face fields per DFT sum, at most
+constexpr int kMarchMinRows = 4;   // rows of a block's chunk, at least
+
+// Several steps of the incident line: from its populations at some time
+// ([Q][n]) to `steps` steps later.  Kept on the way: the moments at the start
+// (lm_from) and after each step (lm[k], [NC][n], E then H components) and the
+// populations after step k (full[k]), each unless NULL.  dft_mask bit k adds
+// the line's field at the pass's k-th time (moments lm_now[k]) to its DFT.
+struct LineMarch {
+    const float *from;
+    int n, steps, axis, w, src_index;
+    float sigma_max, inv_w;
+    float src_E[kMarchSteps][3], src_H[kMarchSteps][3];  // hard-source fields after each step
+    float *lm_from, *lm[kMarchSteps], *full[kMarchSteps];
+    unsigned dft_mask;
+    double dft_scale, dft_c[kMarchSteps], dft_s[kMarchSteps];
+    double *dft;
+    const float *lm_now[kMarchSteps];
+};
+
+// One pass of kMarchSteps steps from time n (times n + 1 + k below).
+struct MarchArgs {
+    const void *fin[14];           // per direction: the pair groups, the singles of level n
+    void *fout[14];                // the same of level n + kMarchSteps
+    const float *inv_eps, *inv_mu; // inv_mu: NULL without a mu_r map
+    int *status;                   // kernel error flags (bit 0: a bounded wait ran out)
+    int nx, ny, nxp;
+    long long P;
+    int strips, rows, line_warps, line_blocks;  // set by the launcher
+    int w;                         // absorbing layer
+    float sigma_max, inv_w;
+    int tfsf, tf_lo[2], tf_hi[2], inc_axis, n_line;
+    const float *lm[kMarchSteps];  // line moments at the fields' times
+    float inv_scale, scale;
+    unsigned dft_mask;             // bit k: the fields of step k are staged at stage[k] ([3][xs_n])
+    float *stage[kMarchSteps];
+    long long xs_n, xs_start[4];
+    int nt_lo[2], nt_hi[2];
+    float *rec[kMarchSteps];       // total-field D (adjoint replay)
+    LineMarch line;                // the line's steps for the next pass (steps = 0: none)
+};
+
+struct DftFlush2dArgs {
+    const float *stage;            // [cnt][3][n]
+    long long n, start[5], plane[4], face_off[4];
+    int cnt;
+    double *dft;
+    double sc[kMarchStage], ss[kMarchStage];
+};
+
+bool march_fits(int mode, int nx, int ny, int nz);
+int line_march_warps(const LineMarch &l);
+// share: how many grids step beside this one
+cudaError_t launch_march(int mode, int storage, const MarchArgs &a, bool rec, int share, cudaStream_t s);
+cudaError_t launch_line_start(int mode, const LineMarch &l, cudaStream_t s);
+cudaError_t launch_dft_flush_2d(const DftFlush2dArgs &a, cudaStream_t s);
 
 // Where the stored populations hold the scattered part G = F - I (inside the
 // total-field box), diagnostics add the incident line back.
