@@ -987,9 +987,23 @@ static int flush_march(lbem_ctx *h)
     return LBEM_OK;
 }
 
-static float *lm_at(lbem_ctx *h, int64_t t)
+// The incident line of a run of 2D passes: its populations by time and the
+// ring of its moments.
+struct LineRun {
+    float *buf[kLineBufs];
+    float *lm;
+    size_t lm_stride;
+    float *at(int64_t t) const { return buf[t % kLineBufs]; }
+    float *moments(int64_t t) const { return lm + (size_t)(t % (2 * kMarchSteps)) * lm_stride; }
+};
+
+static LineRun line_run(lbem_ctx *h)
 {
-    return h->lm + (size_t)(t % (2 * kMarchSteps)) * h->NC * h->n_line_max;
+    LineRun r;
+    for (int k = 0; k < kLineBufs; ++k) r.buf[k] = h->line[k];
+    r.lm = h->lm;
+    r.lm_stride = (size_t)h->NC * h->n_line_max;
+    return r;
 }
 
 // What does not change between a run's passes.
@@ -1039,6 +1053,44 @@ static void march_buffers(MarchArgs &m, const void *in, void *out, size_t plane_
         }
 }
 
+// The line's moments at the times n+1 .. n+K of a pass, from line(n+1), and
+// line(n+K): the start of a run of passes.
+static int march_line_start(lbem_ctx *h, const LineMarch &common, const LineRun &run, int64_t n, const float *from)
+{
+    constexpr int K = kMarchSteps;
+    LineMarch st = common;
+    st.dft_mask = 0;
+    st.from = from;
+    st.steps = K - 1;
+    st.lm_from = run.moments(n + 1);
+    for (int k = 0; k < K; ++k) {
+        st.lm[k] = run.moments(n + 2 + k);
+        st.full[k] = k == K - 2 ? run.at(n + K) : nullptr;
+        source_fields(h, n + 2 + k, st.src_E[k], st.src_H[k]);
+    }
+    CK(h, launch_line_start(h->g.mode, st, h->stream));
+    h->launches += 1;
+    return LBEM_OK;
+}
+
+// The line's part of the pass from time n: the moments it reads, and the
+// line's steps n+K+1 .. n+2K for the next pass.
+static void march_line(lbem_ctx *h, MarchArgs &m, const LineRun &run, int64_t n)
+{
+    constexpr int K = kMarchSteps;
+    LineMarch &l = m.line;
+    l.from = run.at(n + K);
+    l.steps = K;
+    l.dft_mask = 0;
+    for (int k = 0; k < K; ++k) {
+        const int64_t tl = n + K + 1 + k;
+        m.lm[k] = l.lm_now[k] = run.moments(n + 1 + k);
+        l.lm[k] = run.moments(tl);
+        l.full[k] = (k == 0 || k == K - 1) ? run.at(tl) : nullptr;
+        source_fields(h, tl, l.src_E[k], l.src_H[k]);
+    }
+}
+
 // kMarchSteps steps in one pass: level n from f[cur] to f[cur ^ 1].  The pass
 // needs the line's moments at its own times and advances the line for the
 // next one; where the previous pass did not (a first pass, or single steps
@@ -1051,31 +1103,16 @@ static int march_pass(lbem_ctx *h, MarchArgs &m)
     march_buffers(m, h->f[h->cur], h->f[h->cur ^ 1], (size_t)h->P * h->elem);
     m.dft_mask = 0;
     if (h->has_wave) {
-        LineMarch &l = m.line;
+        const LineRun run = line_run(h);
         if (h->line_front != n + K) {
-            LineMarch st = l;
-            st.dft_mask = 0;
-            st.from = line_at(h, n + 1);
-            st.steps = K - 1;
-            st.lm_from = lm_at(h, n + 1);
-            for (int k = 0; k < K; ++k) {
-                st.lm[k] = lm_at(h, n + 2 + k);
-                st.full[k] = k == K - 2 ? line_at(h, n + K) : nullptr;
-                source_fields(h, n + 2 + k, st.src_E[k], st.src_H[k]);
-            }
-            CK(h, launch_line_start(h->g.mode, st, h->stream));
-            h->launches += 1;
+            const int rc = march_line_start(h, m.line, run, n, line_at(h, n + 1));
+            if (rc != LBEM_OK) return rc;
             h->line_front = n + K;
         }
-        l.from = line_at(h, n + K);
-        l.steps = K;
-        l.dft_mask = 0;
+        march_line(h, m, run, n);
+        LineMarch &l = m.line;
         for (int k = 0; k < K; ++k) {
-            const int64_t t = n + 1 + k, tl = n + K + 1 + k;
-            m.lm[k] = l.lm_now[k] = lm_at(h, t);
-            l.lm[k] = lm_at(h, tl);
-            l.full[k] = (k == 0 || k == K - 1) ? line_at(h, tl) : nullptr;
-            source_fields(h, tl, l.src_E[k], l.src_H[k]);
+            const int64_t t = n + 1 + k;
             if (h->ms_n == 0 || h->dft_t0 < 1 || t < h->dft_t0 || t >= h->dft_t0 + (int64_t)h->dft_periods * h->T)
                 continue;
             const double ph = 2.0 * M_PI * (double)(t % h->T) / (double)h->T;
@@ -2013,14 +2050,15 @@ void lbem_destroy(lbem_handle h)
 // ------------------------------------------------------------ adjoint
 // Workspace of lbem_forward_checkpointed / lbem_adjoint:
 //   checkpoints  one per segment of K steps: populations and the three incident-line buffers
-//   replay       two population buffers and three line buffers for the forward replay
+//   replay       two population buffers and the line buffers (and, in 2D, the line's
+//                moments) for the forward replay
 //   mu           two adjoint population buffers
 //   rec          total-field D of every step of one segment (K x NE planes)
 //   G            dJ/dX per DFT entry (DFT array layout)
 //   grad         FP64 accumulator of dJ/d(1/eps_r), one per padded cell
 //   gamma, wts   per-angle sensitivities and weights
 struct AdjLayout {
-    size_t ck0, ck_stride, ck_lines, rf[2], rline[3], mu[2], rec, G, grad, gamma, wts, total;
+    size_t ck0, ck_stride, ck_lines, rf[2], rline[kLineBufs], rlm, mu[2], rec, G, grad, gamma, wts, total;
     int nseg;
 };
 
@@ -2037,7 +2075,8 @@ static AdjLayout adj_layout(const lbem_ctx *h, int64_t n_steps, int K)
     auto take = [&](size_t bytes) { size_t at = o; o = align256(o + bytes); return at; };
     L.ck0 = take(L.ck_stride * (size_t)L.nseg);
     for (int k = 0; k < 2; ++k) L.rf[k] = take(pop);
-    for (int k = 0; k < 3; ++k) L.rline[k] = take(line);
+    for (int k = 0; k < kLineBufs; ++k) L.rline[k] = take(line);
+    L.rlm = take(h->g.mode != 2 ? (size_t)2 * kMarchSteps * h->NC * h->n_line_max * 4 : 0);
     for (int k = 0; k < 2; ++k) L.mu[k] = take(pop);
     L.rec = take((size_t)K * NE * h->P * 4);
     L.G = take(h->dft_doubles_max * 8);
@@ -2195,7 +2234,10 @@ int32_t lbem_adjoint(lbem_handle h, const double *theta, const double *phi, cons
     //    D^F recorded, then the adjoint steps of the segment
     float *mu[2] = {(float *)(W + L.mu[0]), (float *)(W + L.mu[1])};
     float *rf[2] = {(float *)(W + L.rf[0]), (float *)(W + L.rf[1])};
-    float *rline[3] = {(float *)(W + L.rline[0]), (float *)(W + L.rline[1]), (float *)(W + L.rline[2])};
+    LineRun rl;   // the replay's own line
+    for (int k = 0; k < kLineBufs; ++k) rl.buf[k] = (float *)(W + L.rline[k]);
+    rl.lm = (float *)(W + L.rlm);
+    rl.lm_stride = (size_t)h->NC * h->n_line_max;
     float *rec = (float *)(W + L.rec);
     double *grad = (double *)(W + L.grad);
     CK(h, cudaMemsetAsync(mu[0], 0, pop, h->stream));
@@ -2227,6 +2269,35 @@ int32_t lbem_adjoint(lbem_handle h, const double *theta, const double *phi, cons
     }
     b.dft_scale = scale;
 
+    // 2D: passes of kMarchSteps steps, both ways, and single steps for the rest
+    const bool march = march_passes(h);
+    const size_t plane_bytes = (size_t)h->P * 4;
+    MarchArgs m;
+    MarchAdjointArgs mb;
+    if (march) {
+        march_common(h, m);
+        std::memset(&mb, 0, sizeof mb);
+        mb.inv_eps = h->inv_eps;
+        mb.grad = mb.grad_out = grad;
+        mb.status = h->flag + 1;
+        mb.nx = h->g.nx; mb.ny = h->g.ny; mb.nxp = h->nxp;
+        mb.P = h->P;
+        mb.w = b.w;
+        mb.sigma_max = b.sigma_max;
+        mb.inv_w = b.inv_w;
+        mb.dft_scale = scale;
+        mb.G = wa.G;
+        for (int k = 0; k < 2; ++k) {
+            mb.nt_lo[k] = b.nt_lo[k];
+            mb.nt_hi[k] = b.nt_hi[k];
+        }
+        for (int f = 0; f < 4; ++f) {
+            mb.face_off[f] = b.face_off[f];
+            mb.face_nu[f] = b.face_nu[f];
+            mb.face_nv[f] = b.face_nv[f];
+        }
+    }
+
     // phase timing: events before the replay, between replay and backward, after
     std::vector<cudaEvent_t> ev((size_t)3 * L.nseg, nullptr);
     struct EventGuard {
@@ -2238,41 +2309,81 @@ int32_t lbem_adjoint(lbem_handle h, const double *theta, const double *phi, cons
         const int64_t t0 = (int64_t)seg * h->adj_K;
         CK(h, cudaEventRecord(ev[3 * seg], h->stream));
         const int64_t len = std::min<int64_t>(h->adj_K, h->adj_steps - t0);
-        const char *ck = W + L.ck0 + (size_t)seg * L.ck_stride;
-        CK(h, cudaMemcpyAsync(rf[0], ck, pop, cudaMemcpyDeviceToDevice, h->stream));
-        for (int k = 0; k < 3; ++k)
-            CK(h, cudaMemcpyAsync(rline[k], ck + L.ck_lines + k * align256(line), line,
-                                  cudaMemcpyDeviceToDevice, h->stream));
-        for (int64_t k = 0; k < len; ++k) {
+        char *ck = W + L.ck0 + (size_t)seg * L.ck_stride;
+        // the replay reads the segment's first state and line from the checkpoint
+        void *state = ck;
+        int into = 0;            // the buffer the next launch writes
+        auto line_from = [&](int64_t t) {
+            return t <= t0 + 1 ? (float *)(ck + L.ck_lines + (size_t)(t % 3) * align256(line)) : rl.at(t);
+        };
+        int64_t front = -1;
+        for (int64_t k = 0; k < len;) {
             const int64_t t = t0 + k;   // state time before the step
-            for (int q = 0; q < h->Q; ++q) {
-                a.fin_q[q] = rf[k & 1] + (size_t)q * h->P;
-                a.fout_q[q] = rf[(k & 1) ^ 1] + (size_t)q * h->P;
+            if (march && len - k >= kMarchSteps) {
+                if (front != t + kMarchSteps) {
+                    const int rc = march_line_start(h, m.line, rl, t, line_from(t + 1));
+                    if (rc != LBEM_OK) return rc;
+                }
+                march_buffers(m, state, rf[into], plane_bytes);
+                march_line(h, m, rl, t);
+                for (int j = 0; j < kMarchSteps; ++j) m.rec[j] = rec + (size_t)(k + j) * NE * h->P;
+                const cudaError_t e = launch_march(h->g.mode, h->g.storage, m, true, 1, h->stream);
+                if (e != cudaSuccess) return cuda_fail(h, e, "replay pass launch");
+                front = t + 2 * kMarchSteps;
+                k += kMarchSteps;
+            } else {
+                for (int q = 0; q < h->Q; ++q) {
+                    a.fin_q[q] = (const float *)state + (size_t)q * h->P;
+                    a.fout_q[q] = rf[into] + (size_t)q * h->P;
+                }
+                a.line_n = line_from(t);
+                a.line_n1 = line_from(t + 1);
+                a.line_out = rl.at(t + 2);
+                source_fields(h, t + 2, a.src_E, a.src_H);
+                a.rec = rec + (size_t)k * NE * h->P;
+                const cudaError_t e = launch_step_record(h->g.mode, a, h->stream);
+                if (e != cudaSuccess) return cuda_fail(h, e, "replay step launch");
+                k += 1;
             }
-            a.line_n = rline[t % 3];
-            a.line_n1 = rline[(t + 1) % 3];
-            a.line_out = rline[(t + 2) % 3];
-            source_fields(h, t + 2, a.src_E, a.src_H);
-            a.rec = rec + (size_t)k * NE * h->P;
-            cudaError_t e = launch_step_record(h->g.mode, a, h->stream);
-            if (e != cudaSuccess) return cuda_fail(h, e, "replay step launch");
             h->launches += 1;
+            state = rf[into];
+            into ^= 1;
         }
         CK(h, cudaEventRecord(ev[3 * seg + 1], h->stream));
-        for (int64_t k = len - 1; k >= 0; --k) {
-            const int64_t tf = t0 + k + 1;   // time of the fields of this step
-            for (int q = 0; q < h->Q; ++q) {
-                b.lin_q[q] = mu[mcur] + (size_t)q * h->P;
-                b.lout_q[q] = mu[mcur ^ 1] + (size_t)q * h->P;
+        // time tf of a step's fields: whether the DFT window holds it, and its phase
+        auto phase_at = [&](int64_t tf, double &c, double &s) {
+            if (tf < h->dft_t0 || tf > w_end) return false;
+            const double ph = 2.0 * M_PI * (double)(tf % h->T) / (double)h->T;
+            c = std::cos(ph);
+            s = std::sin(ph);
+            return true;
+        };
+        for (int64_t k = len - 1; k >= 0;) {
+            cudaError_t e;
+            if (march && k + 1 >= kMarchSteps) {
+                for (int i = 0; i < 7; ++i)
+                    for (int j = 0; j < 2; ++j) {
+                        const size_t at = (size_t)(3 * i + 2 * j) * h->P;
+                        mb.lin[2 * i + j] = mu[mcur] + at;
+                        mb.lout[2 * i + j] = mu[mcur ^ 1] + at;
+                    }
+                mb.dft_mask = 0;
+                for (int j = 0; j < kMarchSteps; ++j) {
+                    mb.rec[j] = rec + (size_t)(k - j) * NE * h->P;
+                    if (phase_at(t0 + k - j + 1, mb.dft_c[j], mb.dft_s[j])) mb.dft_mask |= 1u << j;
+                }
+                e = launch_march_adjoint(h->g.mode, mb, h->stream);
+                k -= kMarchSteps;
+            } else {
+                for (int q = 0; q < h->Q; ++q) {
+                    b.lin_q[q] = mu[mcur] + (size_t)q * h->P;
+                    b.lout_q[q] = mu[mcur ^ 1] + (size_t)q * h->P;
+                }
+                b.rec = rec + (size_t)k * NE * h->P;
+                b.dft_on = phase_at(t0 + k + 1, b.dft_c, b.dft_s);
+                e = launch_adjoint_step(h->g.mode, b, h->stream);
+                k -= 1;
             }
-            b.rec = rec + (size_t)k * NE * h->P;
-            b.dft_on = tf >= h->dft_t0 && tf <= w_end;
-            if (b.dft_on) {
-                const double ph = 2.0 * M_PI * (double)(tf % h->T) / (double)h->T;
-                b.dft_c = std::cos(ph);
-                b.dft_s = std::sin(ph);
-            }
-            cudaError_t e = launch_adjoint_step(h->g.mode, b, h->stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "adjoint step launch");
             h->launches += 1;
             mcur ^= 1;

@@ -517,6 +517,29 @@ struct AdjWeightArgs {
     double *G;                 // output, DFT layout
 };
 
+// Four backward steps in one 2D pass (march_adjoint.cu), the k-th of them with
+// the DFT phase dft_c[k], dft_s[k] and the recorded D rec[k] of its own step.
+struct MarchAdjointArgs {
+    const float *lin[14];          // per direction: the pair groups, the singles of mu
+    void *lout[14];
+    const float *inv_eps;
+    const float *rec[kMarchSteps];
+    double *grad;                  // read, and written at grad_out (the same array)
+    double *grad_out;
+    int *status;
+    int nx, ny, nxp;
+    long long P;
+    int strips, rows;              // set by the launcher
+    int w;
+    float sigma_max, inv_w;
+    unsigned dft_mask;
+    double dft_c[kMarchSteps], dft_s[kMarchSteps], dft_scale;
+    int nt_lo[2], nt_hi[2];
+    const double *G;
+    long long face_off[4];
+    int face_nu[4], face_nv[4];
+};
+cudaError_t launch_march_adjoint(int mode, const MarchAdjointArgs &a, cudaStream_t s);
 cudaError_t launch_adjoint_step(int mode, const AdjointArgs &a, cudaStream_t s);
 cudaError_t launch_adjoint_weights(const AdjWeightArgs &a, cudaStream_t s, int *launches);
 cudaError_t launch_adjoint_finalize(const double *grad, const float *inv_eps, int nx, int ny, int nz,

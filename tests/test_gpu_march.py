@@ -88,3 +88,35 @@ def test_line_restarts_after_a_snapshot():
     lbem.lbem_load_state(s.h, snap)
     s.step(60)
     assert np.array_equal(s.populations(), ref)
+
+
+@pytest.mark.parametrize("mode", ["ez", "hz"])
+@pytest.mark.parametrize("nx,ny,K", [(57, 61, 23), (113, 300, 31), (168, 50, 20), (600, 53, 25)])
+def test_adjoint_passes_match_single_steps(mode, nx, ny, K):
+    """Replay and backward sweep in passes of four steps (with the single steps
+    that K leaves over) against one launch a step.  The arithmetic is the same
+    but for the FP64 phase products of the DFT source, whose contraction the
+    compiler chooses: a difference of 2^-52 there can move its FP32 rounding by
+    one unit (6e-8), and the sweep is linear in it; 1e-6 allows sixteen of them."""
+    from paper_2510_11042_gb300 import lbem
+    import torch
+    w = 5
+    wv = W.axis_wave(mode, (nx, ny, 1), w, 6.0, gap_ntff=2, gap_tf=2)
+    eps = np.ones((1, ny, nx), np.float32)
+    eps[0, ny // 2 - 6:ny // 2 + 6, wv.tf_lo[0] + 2:wv.tf_lo[0] + 14] = W.random_eps((12, 12, 1), 1.5, 3.0, 4)[0]
+    steps = 3 * nx // 2 + 150
+    p = W.Problem("adj_march", mode, (nx, ny, 1), eps, w, 0.3, wv, steps, 1)
+    got = []
+    for fuse in (1, 2):
+        s = gpu_solver(p, steps=0)
+        s.set_step_fusion(fuse)
+        s.set_dft_window(steps - 17, 1)
+        s.forward_checkpointed(steps, K)
+        J, g = s.adjoint([0.0, 1.0], None, [1.0, 0.5])
+        got.append((J, g.cpu().numpy()))
+        torch.cuda.synchronize()
+        s.close()
+    (j0, g0), (j1, g1) = got
+    assert j0 > 0 and np.abs(g0).max() > 0
+    assert abs(j1 - j0) <= 1e-12 * j0
+    assert np.linalg.norm(g1 - g0) <= 1e-6 * np.linalg.norm(g0)
