@@ -105,12 +105,24 @@ __device__ __forceinline__ void aa_store_dir(void *const *b, int k, void *fb, in
 #undef SQ
 }
 
+// Whether the update tests for source and layer one by one (16-bit BF16) or
+// leaves before them, and the resident blocks per SM the 3D kernel is compiled
+// for: these kernels wait on their loads, and what serves them best depends on
+// how the compiler schedules these around the update (300^3 in the DFT window,
+// us a step, [late, 7 / 8 blocks; early, 7 / 8]: BF16 [876 / 814; 876 / 850],
+// FP16 [849 / 847; 820 / 839], FP32 [1464 / 1360; 1369 / 1360]).
+template <class S> __host__ __device__ constexpr bool aa_late() { return std::is_same<S, __nv_bfloat16>::value; }
+template <int MODE, class S, bool ANA> constexpr int aa_blocks()
+{
+    return MODE != 2 ? 7 : (ANA ? 5 : (std::is_same<S, __half>::value ? 7 : 8));
+}
+
 // One row tile of cells for one step of the given kind (0 push, 1 in place).
 // The host points the group pointers so that the kernel sees its own slot i
 // where the scheme puts direction i: the push step writes direction i through
 // fout_q (aimed at slot opp(i)) and the in-place step reads it through fin_q
 // (aimed at slot opp(i)).
-template <int MODE, class S, int BX, bool MU, bool ANA, int KIND>
+template <int MODE, class S, int BX, bool MU, bool ANA, int KIND, int FORM>
 __device__ __forceinline__ void aa_row(const StepArgs &a, const AaArgs &g, int bx, int y, int z)
 {
     constexpr int Q = Planes<MODE>::Q;
@@ -136,7 +148,7 @@ __device__ __forceinline__ void aa_row(const StepArgs &a, const AaArgs &g, int b
         }
     }
     FloatCell cell{f};
-    update_cell<MODE, false, MU, ANA>(cell, x, y, z, __ldg(a.inv_eps + c), a, MU ? __ldg(a.inv_mu + c) : 1.0f);
+    update_cell<MODE, false, MU, ANA, FORM, !aa_late<S>()>(cell, x, y, z, __ldg(a.inv_eps + c), a, MU ? __ldg(a.inv_mu + c) : 1.0f);
     aa_store_dir<MODE, S>(a.fout_q, c, nullptr, 0, 0, false, 0, f);
 #pragma unroll
     for (int i = 1; i < 7; ++i) {
@@ -162,8 +174,8 @@ __device__ __forceinline__ void aa_row(const StepArgs &a, const AaArgs &g, int b
 // on GB300, several rows per block made the push step of 16-bit storage 20%
 // slower and gained nothing in FP32); the first blocks also update the
 // incident line.
-template <int MODE, class S, int BX, bool MU, bool ANA, int KIND>
-__global__ void __launch_bounds__(BX, (ANA && MODE == 2) ? 5 : 7) aa_step_kernel(const StepArgs a, const AaArgs g)
+template <int MODE, class S, int BX, bool MU, bool ANA, int KIND, int FORM>
+__global__ void __launch_bounds__(BX, (aa_blocks<MODE, S, ANA>())) aa_step_kernel(const StepArgs a, const AaArgs g)
 {
     const int b = blockIdx.x;
     if (a.line_on) {
@@ -171,7 +183,7 @@ __global__ void __launch_bounds__(BX, (ANA && MODE == 2) ? 5 : 7) aa_step_kernel
         if (s < a.n_line) line_work<MODE>(a, s);
     }
     const int r = b / a.nblk_x;
-    aa_row<MODE, S, BX, MU, ANA, KIND>(a, g, b % a.nblk_x, r % a.ny, r / a.ny);
+    aa_row<MODE, S, BX, MU, ANA, KIND, FORM>(a, g, b % a.nblk_x, r % a.ny, r / a.ny);
 }
 
 // The face cell k of axis ax (the other two coordinates, the lower one
@@ -277,7 +289,13 @@ cudaError_t launch_aa_t(StepArgs a, const AaArgs &g, cudaStream_t s)
     if (a.line_on && (a.n_line + kAaBX - 1) / kAaBX > a.nblk_main) return cudaErrorInvalidValue;
     if (MU && a.inv_mu == nullptr) return cudaErrorInvalidValue;
     if (ANA != (a.tfsf == 2)) return cudaErrorInvalidValue;
-    aa_step_kernel<MODE, S, kAaBX, MU, ANA, KIND><<<a.nblk_main, kAaBX, 0, s>>>(a, g);
+    if constexpr (MODE == 2) {
+        if (a.dft_on && !a.xstage) {  // the faces are too large to stage
+            aa_step_kernel<MODE, S, kAaBX, MU, ANA, KIND, kDirect><<<a.nblk_main, kAaBX, 0, s>>>(a, g);
+            return cudaGetLastError();
+        }
+    }
+    aa_step_kernel<MODE, S, kAaBX, MU, ANA, KIND, kStaged><<<a.nblk_main, kAaBX, 0, s>>>(a, g);
     return cudaGetLastError();
 }
 

@@ -60,12 +60,8 @@ struct lbem_ctx {
     float *xstage = nullptr;    // [2][kXBank][NC][xs_n]
     size_t xstage_floats = 0;
     long long xs_n = 0;         // cells of all faces (0: no staging)
-    unsigned xs_xmask = 0;      // the x faces (staged by single steps)
-    unsigned xs_allmask = 0;    // every face (staged by two-step passes)
     int xs_bank = 0;            // the bank being filled
     int xs_cnt = 0;             // its staged steps
-    bool xs_wide = false;       // a step staged faces beyond x that the step stream has not summed
-    unsigned xs_masks[kXBank];
     double xs_sc[kXBank], xs_ss[kXBank];
     // 2D passes of kMarchSteps steps (march.cu): moments of the incident line
     // at 2 kMarchSteps times (time t at t mod that), and the time up to which
@@ -372,6 +368,13 @@ static void fill_common_args(lbem_ctx *h, StepArgs &a)
         a.face_nu[f] = h->faces.nu[f];
         a.face_nv[f] = h->faces.nv[f];
     }
+    for (int ax = 0, f = 0; ax < 3; ++ax) {
+        const bool has = f < h->faces.nfaces && h->faces.axis[f] == ax;
+        a.ft_lo[ax] = has ? a.nt_lo[ax] : -1;
+        a.ft_hi[ax] = has ? a.nt_hi[ax] : -1;
+        for (int k = 0; k < 2 && has; ++k) a.ft_at[ax][k] = (int)h->faces.cell_start[f + k];
+        f += has ? 2 : 0;
+    }
     a.line_dft = h->line_dft;
 }
 
@@ -587,16 +590,13 @@ static void build_faces(lbem_ctx *h)
     }
     F.cell_start[F.nfaces] = cells;
     h->dft_doubles = (size_t)off;
-    // staging in 3D only; faces 0 and 1 are the x faces when the grid has an x extent
+    // staging in banks: 3D
     h->xs_n = (h->g.mode == 2 && F.nfaces > 0) ? (long long)cells : 0;
     if ((size_t)h->xs_n * h->NC * kXStage > h->xstage_floats) h->xs_n = 0;  // cannot happen: bounded by the grid
     // the bank sums index with 32 bits; past that the faces are summed in place
     if ((long long)h->xs_n * h->NC * kXBank > INT_MAX || h->dft_doubles > (size_t)INT_MAX) h->xs_n = 0;
-    h->xs_xmask = (F.nfaces >= 2 && F.axis[0] == 0) ? 3u : 0u;
-    h->xs_allmask = (1u << F.nfaces) - 1u;
     h->xs_bank = 0;
     h->xs_cnt = 0;
-    h->xs_wide = false;
     // 2D: the four faces of a box in x and y
     h->ms_n = (h->g.mode != 2 && F.nfaces == 4) ? cells : 0;
     h->ms_cnt = 0;
@@ -844,7 +844,6 @@ static int flush_x_stage(lbem_ctx *h, bool beside)
         }
         f.start[h->faces.nfaces] = h->faces.cell_start[h->faces.nfaces];
         for (int s = 0; s < h->xs_cnt; ++s) {
-            f.mask[s] = h->xs_masks[s];
             f.sc[s] = h->xs_sc[s];
             f.ss[s] = h->xs_ss[s];
         }
@@ -869,7 +868,6 @@ static int flush_x_stage(lbem_ctx *h, bool beside)
             CK(h, cudaStreamWaitEvent(h->stream, h->xs_summed[b ^ 1], 0));
         }
     }
-    if (!beside) h->xs_wide = false;
     return LBEM_OK;
 }
 
@@ -914,18 +912,15 @@ static void step_args_at(lbem_ctx *h, StepArgs &a, int64_t tn, int in, int out)
     a.xstage = nullptr;
 }
 
-// Claim the next staging slot for a step with the DFT on, staging the faces
-// in mask.
-static void stage_slot(lbem_ctx *h, StepArgs &a, unsigned mask)
+// Claim the next staging slot for a step with the DFT on.
+static void stage_slot(lbem_ctx *h, StepArgs &a)
 {
-    if (!a.dft_on || h->xs_n == 0 || mask == 0) return;
+    if (!a.dft_on || h->xs_n == 0) return;
     a.xstage = h->xstage + ((size_t)h->xs_bank * kXBank + h->xs_cnt) * h->NC * h->xs_n;
     a.xs_n = h->xs_n;
     for (int f = 0; f < h->faces.nfaces; ++f) a.xs_start[f] = h->faces.cell_start[f];
-    h->xs_masks[h->xs_cnt] = mask;
     h->xs_sc[h->xs_cnt] = a.dft_sc;
     h->xs_ss[h->xs_cnt] = a.dft_ss;
-    h->xs_wide = h->xs_wide || (mask & ~h->xs_xmask) != 0;
     ++h->xs_cnt;
 }
 
@@ -1162,7 +1157,9 @@ static int step_loop(lbem_ctx *h, int64_t n)
             k += kMarchSteps;
             continue;
         }
-        if (pairs && n - k >= 2) {
+        // (a two-step pass stages the faces: where they are too large, single
+        // steps add to the accumulators in place)
+        if (pairs && n - k >= 2 && (h->xs_n > 0 || h->faces.nfaces == 0 || h->dft_t0 < 1)) {
             // two steps in one pass: level n from f[cur], level n+2 into f[cur ^ 1]
             if (h->xs_cnt + 2 > kXBank) {
                 const int rc = flush_x_stage(h, true);
@@ -1171,8 +1168,8 @@ static int step_loop(lbem_ctx *h, int64_t n)
             step_args_at(h, a, h->t, h->cur, h->cur ^ 1);
             step_args_at(h, a2, h->t + 1, h->cur ^ 1, h->cur ^ 1);
             const int cnt0 = h->xs_cnt;
-            stage_slot(h, a, h->xs_allmask);
-            stage_slot(h, a2, h->xs_allmask);
+            stage_slot(h, a);
+            stage_slot(h, a2);
             cudaError_t e = launch_step2(h->g.storage, step_variant(h), a, a2, h->stream);
             if (e != cudaSuccess) {
                 h->xs_cnt = cnt0;   // the claimed slots hold nothing
@@ -1183,13 +1180,8 @@ static int step_loop(lbem_ctx *h, int64_t n)
             h->t += 2;
             k += 2;
         } else {
-            // a single step updates the faces it does not stage in place, so
-            // terms staged for them by two-step passes go in first, on the
-            // step stream
-            if (h->xs_wide) {
-                const int rc = flush_x_stage(h, false);
-                if (rc != LBEM_OK) return rc;
-            }
+            // 2D: a single step adds to the accumulators in place, after the
+            // terms that passes have staged
             const int rc2 = flush_march(h);
             if (rc2 != LBEM_OK) return rc2;
             const int kind = h->aa_phase;  // in-place streaming: 0 push, 1 in place
@@ -1206,7 +1198,7 @@ static int step_loop(lbem_ctx *h, int64_t n)
                 step_args_at(h, a, h->t, h->cur, h->cur ^ 1);
             }
             const int cnt0 = h->xs_cnt;
-            stage_slot(h, a, h->xs_xmask);
+            stage_slot(h, a);
             cudaError_t e = h->aa       ? launch_aa_step(h->g.mode, h->g.storage, step_variant(h), kind, a,
                                                          h->aa_g, h->stream)
                             : h->analytic ? launch_step_analytic(h->g.mode, h->g.storage, a, h->stream)

@@ -223,6 +223,9 @@ struct StepArgs {
     float *xstage;             // 3D, non-NULL: staged face fields go here ([NC][xs_n]) for dft_flush_x
     long long xs_n;            // cells of all faces (one component of one staged step)
     long long xs_start[kMaxFaces];  // first staged cell of each face
+    // 3D: the box planes of each axis with faces (-1 for a 1-cell axis, which
+    // has none), and the first staged cell of each face
+    int ft_lo[3], ft_hi[3], ft_at[3][2];
     int nt_lo[3], nt_hi[3];
     double *dft;
     long long face_off[kMaxFaces];
@@ -403,8 +406,7 @@ struct FaceGeom {
 
 // Deferred DFT of NTFF faces: two banks of kXBank steps of staged fields
 // [step][NC][n] (n the cells of all faces, face f from start[f]); one flush
-// sums one bank: the faces each of its steps staged and the steps' phase
-// coefficients.
+// sums one bank of cnt steps with the steps' phase coefficients.
 constexpr int kXBank = 8;
 constexpr int kXStage = 2 * kXBank;
 struct DftFlushArgs {
@@ -415,7 +417,6 @@ struct DftFlushArgs {
     long long start[kMaxFaces + 1];
     long long plane[kMaxFaces];     // nu * nv of each face
     long long face_off[kMaxFaces];
-    unsigned mask[kXBank];
     double sc[kXBank], ss[kXBank];
 };
 // blocks = 0: one thread per summed value; blocks > 0: that many blocks

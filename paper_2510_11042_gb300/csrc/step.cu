@@ -63,7 +63,7 @@ namespace {
 // in-group offset from a constant-bank base; the +-x pulls are plain loads
 // shifted by one element (coalesced; the extra sector per warp hits in L1/L2).
 // The cells x = bx * BX + threadIdx.x of row (y, z) for one step.
-template <int MODE, class S, int BX, bool REC = false, bool MU = false, bool ANA = false>
+template <int MODE, class S, int BX, bool REC = false, bool MU = false, bool ANA = false, int FORM = kStaged>
 __device__ __forceinline__ void row_cells(const StepArgs &a, int bx, int y, int z)
 {
     using PL = Planes<MODE>;
@@ -85,7 +85,7 @@ __device__ __forceinline__ void row_cells(const StepArgs &a, int bx, int y, int 
     float f[Q];
     load_cell<MODE, S>(a, src, f);
     FloatCell cell{f};
-    update_cell<MODE, REC, MU, ANA>(cell, x, y, z, __ldg(a.inv_eps + c), a,
+    update_cell<MODE, REC, MU, ANA, FORM>(cell, x, y, z, __ldg(a.inv_eps + c), a,
                                     MU ? __ldg(a.inv_mu + c) : 1.0f);
     store_cell<MODE, S>(a, c, f);
 }
@@ -101,7 +101,8 @@ __device__ __forceinline__ void row_cells(const StepArgs &a, int bx, int y, int 
 // the 384^3 sphere and 256^2 to 4096^2 EZ grids on GB300.
 template <class S> __host__ __device__ constexpr int rows_of() { return sizeof(S) == 4 ? 2 : 4; }
 
-template <int MODE, class S, int BX, bool REC = false, bool MU = false, bool ANA = false, bool ONE = false>
+template <int MODE, class S, int BX, bool REC = false, bool MU = false, bool ANA = false, bool ONE = false,
+          int FORM = kStaged>
 __global__ void __launch_bounds__(BX, (ANA && MODE == 2) ? 5 : 7) step_kernel_cell(const StepArgs a)
 {
     constexpr int R = ONE ? 1 : rows_of<S>();
@@ -113,7 +114,7 @@ __global__ void __launch_bounds__(BX, (ANA && MODE == 2) ? 5 : 7) step_kernel_ce
     const int bx = b % a.nblk_x;
     const int r0 = (b / a.nblk_x) * R;
     const int r1 = min(r0 + R, a.ny * a.nz);
-    for (int r = r0; r < r1; ++r) row_cells<MODE, S, BX, REC, MU, ANA>(a, bx, r % a.ny, r / a.ny);
+    for (int r = r0; r < r1; ++r) row_cells<MODE, S, BX, REC, MU, ANA, FORM>(a, bx, r % a.ny, r / a.ny);
 }
 
 constexpr int kBX = 128;  // threads per block = cells per row tile
@@ -242,7 +243,7 @@ __global__ void __launch_bounds__(kBX) batch_kernel(const BatchArgs b)
                 const int r0 = (li / sa.nblk_x) * b.rows_per_item;
                 const int bx = li % sa.nblk_x;
                 for (int r = r0; r < min(r0 + b.rows_per_item, rows); ++r)
-                    row_cells<MODE, S, kBX>(sa, bx, r % sa.ny, r / sa.ny);
+                    row_cells<MODE, S, kBX, false, false, false, kDirect>(sa, bx, r % sa.ny, r / sa.ny);
             }
             __syncthreads();
         }
@@ -268,8 +269,7 @@ __global__ void line_init_kernel(const StepArgs a)
 // order, with the same fma as the direct path.  A thread takes one face cell
 // per pass of the grid-stride loop and the components k = blockIdx.y,
 // blockIdx.y + gridDim.y, ...; reads are coalesced along the cells and a
-// component's staged values are all loaded before its FP64 chain.  Slot s
-// holds the faces in mask[s].  A small grid of it (one block per SM, every
+// component's staged values are all loaded before its FP64 chain.  A small grid of it (one block per SM, every
 // component) runs beside the two-step kernel that fills the other bank, one
 // block beside each two-step block: that needs its warps to fit the
 // registers the two-step block leaves on each SM sub-partition (1024 beside
@@ -288,11 +288,6 @@ __global__ void __launch_bounds__(kFlushThreads, 16) dft_flush_x_kernel(const Df
     for (int j = blockIdx.x * kFlushThreads + threadIdx.x; j < n; j += gridDim.x * kFlushThreads) {
         int f = 0;
         while (f + 1 < a.nfaces && j >= a.start[f + 1]) ++f;
-        unsigned on = 0;  // the slots that staged face f
-#pragma unroll
-        for (int s = 0; s < kXBank; ++s)
-            if (s < a.cnt) on |= ((a.mask[s] >> f) & 1u) << s;
-        if (!on) continue;
         const float *src = a.stage + j;
         double *base = a.dft + a.face_off[f] + (j - (int)a.start[f]);
         const int plane = (int)a.plane[f];
@@ -300,11 +295,11 @@ __global__ void __launch_bounds__(kFlushThreads, 16) dft_flush_x_kernel(const Df
             float v[kXBank];
 #pragma unroll
             for (int s = 0; s < kXBank; ++s)
-                v[s] = ((on >> s) & 1u) ? src[s * slot + k * n] : 0.f;
+                v[s] = s < a.cnt ? src[s * slot + k * n] : 0.f;
             double re = base[(2 * k + 0) * plane], im = base[(2 * k + 1) * plane];
 #pragma unroll
             for (int s = 0; s < kXBank; ++s) {
-                if (!((on >> s) & 1u)) continue;
+                if (s >= a.cnt) break;
                 re = fma((double)v[s], a.sc[s], re);
                 im = fma((double)v[s], -a.ss[s], im);
             }
@@ -319,13 +314,20 @@ cudaError_t launch_cell(StepArgs a, cudaStream_t s)
 {
     a.nblk_x = (a.nx + kBX - 1) / kBX;
     a.rows_per_block = rows_of<S>();
-    if ((long long)a.nblk_x * a.ny * a.nz / a.rows_per_block < 7LL * std::max(1, sm_count()))
+    const bool direct = MODE == 2 && a.dft_on && !a.xstage;  // the faces are too large to stage
+    if (direct || (long long)a.nblk_x * a.ny * a.nz / a.rows_per_block < 7LL * std::max(1, sm_count()))
         a.rows_per_block = 1;
     a.nblk_main = a.nblk_x * ((a.ny * a.nz + a.rows_per_block - 1) / a.rows_per_block);
     if (a.line_on && (a.n_line + kBX - 1) / kBX > a.nblk_main) return cudaErrorInvalidValue;
     if (REC && a.rec == nullptr) return cudaErrorInvalidValue;
     if (MU && a.inv_mu == nullptr) return cudaErrorInvalidValue;
     if (ANA != (a.tfsf == 2)) return cudaErrorInvalidValue;
+    if constexpr (MODE == 2 && !REC) {
+        if (direct) {
+            step_kernel_cell<MODE, S, kBX, REC, MU, ANA, true, kDirect><<<a.nblk_main, kBX, 0, s>>>(a);
+            return cudaGetLastError();
+        }
+    }
     if (a.rows_per_block == 1)
         step_kernel_cell<MODE, S, kBX, REC, MU, ANA, true><<<a.nblk_main, kBX, 0, s>>>(a);
     else

@@ -259,13 +259,35 @@ struct FloatCell {
     __device__ __forceinline__ void set(int q, float v) { f[q] = v; }
 };
 
+// The running DFT of cells on the NTFF box, in 3D.  Kernels stage the fields for
+// dft_flush_x: an FP64 read-modify-write in the step holds a warp, and in the
+// two-step kernel a whole tile, for a DRAM round trip and an FP64 pass (64^3
+// FP32 single steps in the window: 23.4 us a step with only the x faces staged,
+// now 15.1).  kStaged tests for a face first and stores straight-line;
+// kStagedByFace loops over the faces, which leaves the issue-bound 16-bit
+// two-step kernel faster (384^3 FP16 outside / in the window 0.896 / 0.957 ms
+// against 0.917 / 0.962; FP32 1.549 / 1.625 against 1.555 / 1.586 the other way).
+// kDirect adds to the accumulators in place: the batched kernel, and grids
+// whose faces are too large to stage -- in a kernel of its own, for with both
+// forms in one the 16-bit single steps spilled (300^3 BF16 in place 778 -> 858 us).
+constexpr int kStaged = 0, kStagedByFace = 1, kDirect = 2;
+
+// The fields of a face cell into its slot of the staged step (element j of
+// xs_n; the host keeps 8 staged steps below 2^31 elements).
+template <int NC> __device__ __forceinline__ void stage_fields(const StepArgs &a, int j, const float vals[NC])
+{
+#pragma unroll
+    for (int k = 0; k < NC; ++k) a.xstage[k * (int)a.xs_n + j] = vals[k];
+}
+
 // Moments, DFT, collision, incident source and absorbing layer of one cell,
 // in one pass over its populations after the moments:
 //   f* = (2 f_eq - f + source) * keep.
 // Values are in storage units (population / scale); fields go to the DFT
 // multiplied back by the scale (dft_scale_cells), the incident source is
 // divided by it.
-template <int MODE, bool REC = false, bool MU = false, bool ANA = false, bool ALLSTAGE = false, class Cell>
+template <int MODE, bool REC = false, bool MU = false, bool ANA = false, int FORM = kStaged, bool EARLY = true,
+          class Cell>
 __device__ __forceinline__ void update_cell(Cell &f, int x, int y, int z, float inv_eps,
                                             const StepArgs &a, float inv_mu = 1.0f, bool surface = true)
 {
@@ -321,58 +343,55 @@ __device__ __forceinline__ void update_cell(Cell &f, int x, int y, int z, float 
         H[c3] = MU ? __fmul_rn(B[c3], inv_mu) : B[c3];
     }
 
-    bool on_face = surface && a.dft_on && in_box(x, y, z, a.nt_lo, a.nt_hi);
-    if constexpr (ALLSTAGE) {
-        // the two-step kernel is issue-bound: keep the cells inside the box out
-        // of the face loop
+    // the running DFT of cells on the NTFF box
+    bool on_face = surface && a.dft_on;
+    if constexpr (MODE == 2 && FORM == kStaged)
+        on_face = on_face && (x == a.ft_lo[0] || x == a.ft_hi[0] || y == a.ft_lo[1] || y == a.ft_hi[1] ||
+                              z == a.ft_lo[2] || z == a.ft_hi[2]);
+    on_face = on_face && in_box(x, y, z, a.nt_lo, a.nt_hi);
+    if constexpr (MODE == 2 && FORM == kStagedByFace)
         on_face = on_face && (x == a.nt_lo[0] || x == a.nt_hi[0] || y == a.nt_lo[1] || y == a.nt_hi[1] ||
                               z == a.nt_lo[2] || z == a.nt_hi[2]);
-    }
     if (on_face) {
-        const int g[3] = {x, y, z};
-        const int n3[3] = {a.nx, a.ny, a.nz};
         float vals[PL::NC];
 #pragma unroll
         for (int k = 0; k < PL::NE; ++k) vals[k] = E[M::ec(k)];
 #pragma unroll
         for (int k = 0; k < PL::NH; ++k) vals[PL::NE + k] = H[M::hc(k)];
-        int face = 0;
-        for (int ax = 0; ax < 3; ++ax) {
-            if (n3[ax] <= 1) continue;
-            for (int side = 0; side < 2; ++side, ++face) {
-                if (g[ax] != (side ? a.nt_hi[ax] : a.nt_lo[ax])) continue;
-                const int ua = ax == 2 ? 1 : 2, va = ax == 0 ? 1 : 0;
-                const int iu = g[ua] - a.nt_lo[ua], iv = g[va] - a.nt_lo[va];
-                const int nu = a.face_nu[face], nv = a.face_nv[face];
-                // Staged faces store the fields and dft_flush_x sums them in full
-                // warps (3D only: in 2D the branch cost more than it saved).  The
-                // single step stages the x faces, which hold two cells per row, one
-                // thread in a warp, whose read-modify-write would hold the warp for
-                // a DRAM round trip and a lone FP64 pass; the two-step kernel
-                // (ALLSTAGE) stages every face, since there the stall would hold
-                // a whole tile at every plane.
-                if constexpr (MODE == 2 && ALLSTAGE) {
-                    if (a.xstage) {
+        if constexpr (MODE == 2 && FORM == kStaged) {
+            const int iu = z - a.nt_lo[2], iy = y - a.nt_lo[1], ix = x - a.nt_lo[0];
+            const int nvx = a.nt_hi[1] - a.nt_lo[1] + 1, nv = a.nt_hi[0] - a.nt_lo[0] + 1;
+            if (x == a.ft_lo[0] || x == a.ft_hi[0])
+                stage_fields<PL::NC>(a, a.ft_at[0][x == a.ft_hi[0]] + iu * nvx + iy, vals);
+            if (y == a.ft_lo[1] || y == a.ft_hi[1])
+                stage_fields<PL::NC>(a, a.ft_at[1][y == a.ft_hi[1]] + iu * nv + ix, vals);
+            if (z == a.ft_lo[2] || z == a.ft_hi[2])
+                stage_fields<PL::NC>(a, a.ft_at[2][z == a.ft_hi[2]] + iy * nv + ix, vals);
+        } else {
+            const int g[3] = {x, y, z};
+            const int n3[3] = {a.nx, a.ny, a.nz};
+            int face = 0;
+            for (int ax = 0; ax < 3; ++ax) {
+                if (n3[ax] <= 1) continue;
+                for (int side = 0; side < 2; ++side, ++face) {
+                    if (g[ax] != (side ? a.nt_hi[ax] : a.nt_lo[ax])) continue;
+                    const int ua = ax == 2 ? 1 : 2, va = ax == 0 ? 1 : 0;
+                    const int iu = g[ua] - a.nt_lo[ua], iv = g[va] - a.nt_lo[va];
+                    const int nu = a.face_nu[face], nv = a.face_nv[face];
+                    if constexpr (MODE == 2 && FORM == kStagedByFace) {
                         const long long j = a.xs_start[face] + (long long)iu * nv + iv;
 #pragma unroll
                         for (int k = 0; k < PL::NC; ++k) a.xstage[(long long)k * a.xs_n + j] = vals[k];
                         continue;
                     }
-                } else if constexpr (MODE == 2) {
-                    if (ax == 0 && a.xstage) {
-                        const long long j = ((long long)side * nu + iu) * nv + iv;
+                    double *base = a.dft + a.face_off[face] + (long long)iu * nv + iv;
+                    const long long plane = (long long)nu * nv;
 #pragma unroll
-                        for (int k = 0; k < PL::NC; ++k) a.xstage[(long long)k * a.xs_n + j] = vals[k];
-                        continue;
+                    for (int k = 0; k < PL::NC; ++k) {
+                        const double v = (double)vals[k];
+                        base[(2 * k + 0) * plane] = fma(v, a.dft_sc, base[(2 * k + 0) * plane]);
+                        base[(2 * k + 1) * plane] = fma(v, -a.dft_ss, base[(2 * k + 1) * plane]);
                     }
-                }
-                double *base = a.dft + a.face_off[face] + (long long)iu * nv + iv;
-                const long long plane = (long long)nu * nv;
-#pragma unroll
-                for (int k = 0; k < PL::NC; ++k) {
-                    const double v = (double)vals[k];
-                    base[(2 * k + 0) * plane] = fma(v, a.dft_sc, base[(2 * k + 0) * plane]);
-                    base[(2 * k + 1) * plane] = fma(v, -a.dft_ss, base[(2 * k + 1) * plane]);
                 }
             }
         }
@@ -394,33 +413,31 @@ __device__ __forceinline__ void update_cell(Cell &f, int x, int y, int z, float 
     const bool source = a.tfsf == 1 && (inv_eps != 1.0f || (MU && inv_mu != 1.0f)) &&
                         in_box(x, y, z, a.tf_lo, a.tf_hi);
     const bool ana = ANA && in_box(x, y, z, a.tf_lo, a.tf_hi);
-    if (!source && !ana && keep == 1.0f) {
-        // most cells: plain collision, f* = 2 f_eq - f
-        if constexpr (MODE == 2) {
-            // in packed pairs (e_x e_y), (e_z h_x), (h_y h_z) per direction:
-            // 2 f_eq + (-1) f rounds once, as 2 f_eq - f does
-            const float2 m1 = make_float2(-1.f, -1.f);
+    // plain collision, f* = 2 f_eq - f
+    if constexpr (MODE == 2) {
+        // in packed pairs (e_x e_y), (e_z h_x), (h_y h_z) per direction:
+        // 2 f_eq + (-1) f rounds once, as 2 f_eq - f does
+        const float2 m1 = make_float2(-1.f, -1.f);
 #pragma unroll
-            for (int i = 0; i < 7; ++i) {
-                float eq[6];
+        for (int i = 0; i < 7; ++i) {
+            float eq[6];
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    eq[k] = (i == 0) ? 2.f * (D[k] - E[k]) : E3[k] - cross_c(i, H3, k);
-                    eq[3 + k] = (i == 0) ? (MU ? 2.f * (B[k] - H[k]) : 0.f) : H3[k] + cross_c(i, E3, k);
-                }
-                const int qe = 3 * i, qh = 21 + 3 * i;
-                const float2 r0 = __ffma2_rn(make_float2(f.get(qe), f.get(qe + 1)), m1, make_float2(eq[0], eq[1]));
-                const float2 r1 = __ffma2_rn(make_float2(f.get(qe + 2), f.get(qh)), m1, make_float2(eq[2], eq[3]));
-                const float2 r2 = __ffma2_rn(make_float2(f.get(qh + 1), f.get(qh + 2)), m1, make_float2(eq[4], eq[5]));
-                f.set(qe, r0.x);
-                f.set(qe + 1, r0.y);
-                f.set(qe + 2, r1.x);
-                f.set(qh, r1.y);
-                f.set(qh + 1, r2.x);
-                f.set(qh + 2, r2.y);
+            for (int k = 0; k < 3; ++k) {
+                eq[k] = (i == 0) ? 2.f * (D[k] - E[k]) : E3[k] - cross_c(i, H3, k);
+                eq[3 + k] = (i == 0) ? (MU ? 2.f * (B[k] - H[k]) : 0.f) : H3[k] + cross_c(i, E3, k);
             }
-            return;
+            const int qe = 3 * i, qh = 21 + 3 * i;
+            const float2 r0 = __ffma2_rn(make_float2(f.get(qe), f.get(qe + 1)), m1, make_float2(eq[0], eq[1]));
+            const float2 r1 = __ffma2_rn(make_float2(f.get(qe + 2), f.get(qh)), m1, make_float2(eq[2], eq[3]));
+            const float2 r2 = __ffma2_rn(make_float2(f.get(qh + 1), f.get(qh + 2)), m1, make_float2(eq[4], eq[5]));
+            f.set(qe, r0.x);
+            f.set(qe + 1, r0.y);
+            f.set(qe + 2, r1.x);
+            f.set(qh, r1.y);
+            f.set(qh + 1, r2.x);
+            f.set(qh + 2, r2.y);
         }
+    } else {
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             const int i = PL::dir(q), ac = PL::comp(q);
@@ -429,15 +446,17 @@ __device__ __forceinline__ void update_cell(Cell &f, int x, int y, int z, float 
             else eq2 = (i == 0) ? (MU ? 2.f * (B[ac] - H[ac]) : 0.f) : H3[ac] + cross_c(i, E3, ac);
             f.set(q, eq2 - f.get(q));
         }
-        return;
     }
-    AnaTerms<MODE> at;
-    if constexpr (ANA) {
-        if (ana) analytic_prepare<MODE>(a, x, y, z, inv_eps, inv_mu, keep, at);
-    }
-    float dE[3] = {0.f, 0.f, 0.f}, dE3[3] = {0.f, 0.f, 0.f};
-    float dH[3] = {0.f, 0.f, 0.f}, dH3[3] = {0.f, 0.f, 0.f};
+    // then the source, the layer and the closed-form source, each where a cell
+    // has it: (f* + src) keep rounds as it does in one expression.  One general
+    // path beside the plain one cost the cells of the absorbing layer, a quarter
+    // of the 384^3 grid, twice the plain update's instructions (two-step passes
+    // at 384^3 in the DFT window: FP32 1.586 -> 1.551 ms, FP16 0.962 -> 0.911).
+    // EARLY leaves before the three tests.
+    if (EARLY && !source && !ana && keep == 1.0f) return;
     if (source) {
+        float dE[3] = {0.f, 0.f, 0.f}, dE3[3] = {0.f, 0.f, 0.f};
+        float dH[3] = {0.f, 0.f, 0.f}, dH3[3] = {0.f, 0.f, 0.f};
         const int sl = a.inc_axis == 0 ? x : (a.inc_axis == 1 ? y : z);
 #pragma unroll
         for (int q = 0; q < 7 * PL::NE; ++q)
@@ -459,25 +478,26 @@ __device__ __forceinline__ void update_cell(Cell &f, int x, int y, int z, float 
                 dH3[c3] = third(dH[c3]);
             }
         }
-    }
-
 #pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        const int i = PL::dir(q), ac = PL::comp(q);
-        float eq2, src;  // 2 f_eq and the incident source
-        if (PL::fam(q) == 0) {
-            eq2 = (i == 0) ? 2.f * (D[ac] - E[ac]) : E3[ac] - cross_c(i, H3, ac);
-            src = (i == 0) ? -2.f * dE[ac] : (MU ? dE3[ac] - cross_c(i, dH3, ac) : dE3[ac]);
-        } else {
-            eq2 = (i == 0) ? (MU ? 2.f * (B[ac] - H[ac]) : 0.f) : H3[ac] + cross_c(i, E3, ac);
-            src = (i == 0) ? (MU ? -2.f * dH[ac] : 0.f)
-                           : (MU ? dH3[ac] + cross_c(i, dE3, ac) : cross_c(i, dE3, ac));
+        for (int q = 0; q < Q; ++q) {
+            const int i = PL::dir(q), ac = PL::comp(q);
+            float src;
+            if (PL::fam(q) == 0) src = (i == 0) ? -2.f * dE[ac] : (MU ? dE3[ac] - cross_c(i, dH3, ac) : dE3[ac]);
+            else src = (i == 0) ? (MU ? -2.f * dH[ac] : 0.f) : (MU ? dH3[ac] + cross_c(i, dE3, ac) : cross_c(i, dE3, ac));
+            f.set(q, f.get(q) + src);
         }
-        float v = (eq2 - f.get(q) + src) * keep;
-        if constexpr (ANA) {
-            if (ana) v += analytic_term<MODE>(a, at, q);
+    }
+    if (keep != 1.0f) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) f.set(q, f.get(q) * keep);
+    }
+    if constexpr (ANA) {
+        if (ana) {
+            AnaTerms<MODE> at;
+            analytic_prepare<MODE>(a, x, y, z, inv_eps, inv_mu, keep, at);
+#pragma unroll
+            for (int q = 0; q < Q; ++q) f.set(q, f.get(q) + analytic_term<MODE>(a, at, q));
         }
-        f.set(q, v);
     }
 }
 
