@@ -126,7 +126,7 @@ template <int MODE, class S, int BX, bool MU, bool ANA, int KIND, int FORM>
 __device__ __forceinline__ void aa_row(const StepArgs &a, const AaArgs &g, int bx, int y, int z)
 {
     constexpr int Q = Planes<MODE>::Q;
-    const int x = bx * BX + threadIdx.x;
+    const int x = bx * blockDim.x + threadIdx.x;
     if (x >= a.nx) return;
     const int pz = a.ny * a.nxp;
     const int c = z * pz + y * a.nxp + x;
@@ -170,7 +170,7 @@ __device__ __forceinline__ void aa_row(const StepArgs &a, const AaArgs &g, int b
     }
 }
 
-// One block per row tile of BX cells (one row per block: measured at 384^3
+// One block per row tile (one row per block: measured at 384^3
 // on GB300, several rows per block made the push step of 16-bit storage 20%
 // slower and gained nothing in FP32); the first blocks also update the
 // incident line.
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(BX, (aa_blocks<MODE, S, ANA>())) aa_step_kerne
 {
     const int b = blockIdx.x;
     if (a.line_on) {
-        const int s = b * BX + threadIdx.x;
+        const int s = b * blockDim.x + threadIdx.x;
         if (s < a.n_line) line_work<MODE>(a, s);
     }
     const int r = b / a.nblk_x;
@@ -276,26 +276,27 @@ __global__ void aa_canon_swap_kernel(T *buf, int mode, int elem, long long P, in
     }
 }
 
-constexpr int kAaBX = 128;  // threads per block = cells per row tile
+constexpr int kAaBX = 128;  // threads per block at most (row_threads)
 
 template <int MODE, class S, bool MU, bool ANA, int KIND>
 cudaError_t launch_aa_t(StepArgs a, const AaArgs &g, cudaStream_t s)
 {
-    a.nblk_x = (a.nx + kAaBX - 1) / kAaBX;
+    const int tx = row_threads(a.nx);
+    a.nblk_x = (a.nx + tx - 1) / tx;
     a.rows_per_block = 1;
     const long long blocks = (long long)a.nblk_x * a.ny * a.nz;
     if (blocks > INT_MAX) return cudaErrorInvalidValue;
     a.nblk_main = (int)blocks;
-    if (a.line_on && (a.n_line + kAaBX - 1) / kAaBX > a.nblk_main) return cudaErrorInvalidValue;
+    if (a.line_on && (a.n_line + tx - 1) / tx > a.nblk_main) return cudaErrorInvalidValue;
     if (MU && a.inv_mu == nullptr) return cudaErrorInvalidValue;
     if (ANA != (a.tfsf == 2)) return cudaErrorInvalidValue;
     if constexpr (MODE == 2) {
         if (a.dft_on && !a.xstage) {  // the faces are too large to stage
-            aa_step_kernel<MODE, S, kAaBX, MU, ANA, KIND, kDirect><<<a.nblk_main, kAaBX, 0, s>>>(a, g);
+            aa_step_kernel<MODE, S, kAaBX, MU, ANA, KIND, kDirect><<<a.nblk_main, tx, 0, s>>>(a, g);
             return cudaGetLastError();
         }
     }
-    aa_step_kernel<MODE, S, kAaBX, MU, ANA, KIND, kStaged><<<a.nblk_main, kAaBX, 0, s>>>(a, g);
+    aa_step_kernel<MODE, S, kAaBX, MU, ANA, KIND, kStaged><<<a.nblk_main, tx, 0, s>>>(a, g);
     return cudaGetLastError();
 }
 

@@ -32,7 +32,7 @@
 // (A and D^F are FP32) and summed over the steps in FP64.
 #include <algorithm>
 
-#include "lbem_internal.cuh"
+#include "step_cell.cuh"
 
 namespace lbem {
 namespace {
@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(kAdjBX, MODE == 2 ? 7 : 1) adjoint_step_kernel
     const int bx = b % a.nblk_x;
     const int row = b / a.nblk_x;
     const int y = row % a.ny, z = row / a.ny;
-    const int x = bx * kAdjBX + threadIdx.x;
+    const int x = bx * blockDim.x + threadIdx.x;
     if (x >= a.nx) return;
     const int pz = a.ny * a.nxp;
     const int c = z * pz + y * a.nxp + x;
@@ -327,10 +327,11 @@ __global__ void adjoint_finalize_kernel(const double *grad, const float *inv_eps
 template <int MODE>
 cudaError_t launch_adj(AdjointArgs a, cudaStream_t s)
 {
-    a.nblk_x = (a.nx + kAdjBX - 1) / kAdjBX;
+    const int tx = row_threads(a.nx);
+    a.nblk_x = (a.nx + tx - 1) / tx;
     const long long blocks = (long long)a.nblk_x * a.ny * a.nz;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    adjoint_step_kernel<MODE><<<(unsigned)blocks, kAdjBX, 0, s>>>(a);
+    adjoint_step_kernel<MODE><<<(unsigned)blocks, tx, 0, s>>>(a);
     return cudaGetLastError();
 }
 

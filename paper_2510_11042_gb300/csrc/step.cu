@@ -62,13 +62,13 @@ namespace {
 // a.fin_q[i * NC + s0] (kernel parameters), so every access is a 32-bit
 // in-group offset from a constant-bank base; the +-x pulls are plain loads
 // shifted by one element (coalesced; the extra sector per warp hits in L1/L2).
-// The cells x = bx * BX + threadIdx.x of row (y, z) for one step.
+// The cells x = bx * blockDim.x + threadIdx.x of row (y, z) for one step.
 template <int MODE, class S, int BX, bool REC = false, bool MU = false, bool ANA = false, int FORM = kStaged>
 __device__ __forceinline__ void row_cells(const StepArgs &a, int bx, int y, int z)
 {
     using PL = Planes<MODE>;
     constexpr int Q = PL::Q;
-    const int x = bx * BX + threadIdx.x;
+    const int x = bx * blockDim.x + threadIdx.x;
     if (x >= a.nx) return;
 
     const int pz = a.ny * a.nxp;
@@ -90,7 +90,7 @@ __device__ __forceinline__ void row_cells(const StepArgs &a, int bx, int y, int 
     store_cell<MODE, S>(a, c, f);
 }
 
-// One block per tile of BX cells x R consecutive rows (y fastest, then z);
+// One block per tile of row_threads(nx) cells x R consecutive rows (y fastest, then z);
 // the first blocks also update the incident line.  R = rows_of<S> blocks of
 // several rows cut the per-block start-up cost of short 128-cell rows; grids
 // of under one wave of such blocks (7 per SM) take one row per block
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(BX, (ANA && MODE == 2) ? 5 : 7) step_kernel_ce
     constexpr int R = ONE ? 1 : rows_of<S>();
     const int b = blockIdx.x;
     if (a.line_on) {
-        const int s = b * BX + threadIdx.x;
+        const int s = b * blockDim.x + threadIdx.x;
         if (s < a.n_line) line_work<MODE>(a, s);
     }
     const int bx = b % a.nblk_x;
@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(BX, (ANA && MODE == 2) ? 5 : 7) step_kernel_ce
     for (int r = r0; r < r1; ++r) row_cells<MODE, S, BX, REC, MU, ANA, FORM>(a, bx, r % a.ny, r / a.ny);
 }
 
-constexpr int kBX = 128;  // threads per block = cells per row tile
+constexpr int kBX = 128;  // threads per block at most; cells per row tile of the batched kernel
 
 // ---------------------------------------------------------------------------
 // Batched persistent kernel: many problems (same mode and storage, any sizes,
@@ -312,26 +312,27 @@ __global__ void __launch_bounds__(kFlushThreads, 16) dft_flush_x_kernel(const Df
 template <int MODE, class S, bool REC = false, bool MU = false, bool ANA = false>
 cudaError_t launch_cell(StepArgs a, cudaStream_t s)
 {
-    a.nblk_x = (a.nx + kBX - 1) / kBX;
+    const int tx = row_threads(a.nx);
+    a.nblk_x = (a.nx + tx - 1) / tx;
     a.rows_per_block = rows_of<S>();
     const bool direct = MODE == 2 && a.dft_on && !a.xstage;  // the faces are too large to stage
     if (direct || (long long)a.nblk_x * a.ny * a.nz / a.rows_per_block < 7LL * std::max(1, sm_count()))
         a.rows_per_block = 1;
     a.nblk_main = a.nblk_x * ((a.ny * a.nz + a.rows_per_block - 1) / a.rows_per_block);
-    if (a.line_on && (a.n_line + kBX - 1) / kBX > a.nblk_main) return cudaErrorInvalidValue;
+    if (a.line_on && (a.n_line + tx - 1) / tx > a.nblk_main) return cudaErrorInvalidValue;
     if (REC && a.rec == nullptr) return cudaErrorInvalidValue;
     if (MU && a.inv_mu == nullptr) return cudaErrorInvalidValue;
     if (ANA != (a.tfsf == 2)) return cudaErrorInvalidValue;
     if constexpr (MODE == 2 && !REC) {
         if (direct) {
-            step_kernel_cell<MODE, S, kBX, REC, MU, ANA, true, kDirect><<<a.nblk_main, kBX, 0, s>>>(a);
+            step_kernel_cell<MODE, S, kBX, REC, MU, ANA, true, kDirect><<<a.nblk_main, tx, 0, s>>>(a);
             return cudaGetLastError();
         }
     }
     if (a.rows_per_block == 1)
-        step_kernel_cell<MODE, S, kBX, REC, MU, ANA, true><<<a.nblk_main, kBX, 0, s>>>(a);
+        step_kernel_cell<MODE, S, kBX, REC, MU, ANA, true><<<a.nblk_main, tx, 0, s>>>(a);
     else
-        step_kernel_cell<MODE, S, kBX, REC, MU, ANA, false><<<a.nblk_main, kBX, 0, s>>>(a);
+        step_kernel_cell<MODE, S, kBX, REC, MU, ANA, false><<<a.nblk_main, tx, 0, s>>>(a);
     return cudaGetLastError();
 }
 
