@@ -178,6 +178,8 @@ template <int MODE, class S, int BX, bool MU, bool ANA, int KIND, int FORM>
 __global__ void __launch_bounds__(BX, (aa_blocks<MODE, S, ANA>())) aa_step_kernel(const StepArgs a, const AaArgs g)
 {
     const int b = blockIdx.x;
+    chain_release();
+    chain_wait();
     if (a.line_on) {
         const int s = b * blockDim.x + threadIdx.x;
         if (s < a.n_line) line_work<MODE>(a, s);
@@ -292,12 +294,10 @@ cudaError_t launch_aa_t(StepArgs a, const AaArgs &g, cudaStream_t s)
     if (ANA != (a.tfsf == 2)) return cudaErrorInvalidValue;
     if constexpr (MODE == 2) {
         if (a.dft_on && !a.xstage) {  // the faces are too large to stage
-            aa_step_kernel<MODE, S, kAaBX, MU, ANA, KIND, kDirect><<<a.nblk_main, tx, 0, s>>>(a, g);
-            return cudaGetLastError();
+            return launch_chained(a.chain != 0, aa_step_kernel<MODE, S, kAaBX, MU, ANA, KIND, kDirect>, a.nblk_main, tx, 0, s, a, g);
         }
     }
-    aa_step_kernel<MODE, S, kAaBX, MU, ANA, KIND, kStaged><<<a.nblk_main, tx, 0, s>>>(a, g);
-    return cudaGetLastError();
+    return launch_chained(a.chain != 0, aa_step_kernel<MODE, S, kAaBX, MU, ANA, KIND, kStaged>, a.nblk_main, tx, 0, s, a, g);
 }
 
 template <int MODE, class S>

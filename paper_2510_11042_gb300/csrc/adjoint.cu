@@ -54,6 +54,8 @@ __global__ void __launch_bounds__(kAdjBX, MODE == 2 ? 7 : 1) adjoint_step_kernel
     using M = Mode<MODE>;
     constexpr int Q = PL::Q;
     const int b = blockIdx.x;
+    chain_release();
+    chain_wait();
     const int bx = b % a.nblk_x;
     const int row = b / a.nblk_x;
     const int y = row % a.ny, z = row / a.ny;
@@ -331,8 +333,7 @@ cudaError_t launch_adj(AdjointArgs a, cudaStream_t s)
     a.nblk_x = (a.nx + tx - 1) / tx;
     const long long blocks = (long long)a.nblk_x * a.ny * a.nz;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    adjoint_step_kernel<MODE><<<(unsigned)blocks, tx, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(chain_pays(a.nx, a.ny, a.nz), adjoint_step_kernel<MODE>, (unsigned)blocks, tx, 0, s, a);
 }
 
 }  // namespace

@@ -338,6 +338,7 @@ static void fill_common_args(lbem_ctx *h, StepArgs &a)
     a.scale = h->scale;
     a.inv_scale = h->inv_scale;
     a.status = h->flag + 1;
+    a.chain = h->share == 1 && chain_pays(a.nx, a.ny, a.nz);
     if (!h->has_wave) return;
     a.tfsf = h->analytic ? 2 : 1;
     a.line_on = h->analytic ? 0 : 1;

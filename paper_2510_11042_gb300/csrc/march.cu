@@ -315,7 +315,9 @@ __global__ void __launch_bounds__(32 * kRows, 16 / kRows) march_kernel(const __g
     using Y = YBuf<S>;
     extern __shared__ __align__(16) unsigned char ybuf[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    chain_release();
     if ((int)blockIdx.x < a.line_blocks) {
+        chain_wait();
         const int k = blockIdx.x * kRows + w;
         if (k < a.line_warps) line_march<MODE>(a.line, k);
         return;
@@ -330,6 +332,7 @@ __global__ void __launch_bounds__(32 * kRows, 16 / kRows) march_kernel(const __g
     const int pa = max(y0 - (K - 1), 0), pend = min(y1 - 1 + (K - 1), a.ny - 1);
     __shared__ __align__(8) unsigned long long done[kRows][K];
     init_rows(done);
+    chain_wait();
 
     Dir2<S> d[7];               // this warp's row, in storage form between levels
     P2 ie = both(1.f), im = both(1.f);
@@ -435,8 +438,7 @@ cudaError_t launch_march_t(MarchArgs a, int share, cudaStream_t s)
     a.line_blocks = (a.line_warps + kRows - 1) / kRows;
     const long long blocks = a.line_blocks + chunks * a.strips;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    march_kernel<MODE, S, MU, REC><<<(unsigned)blocks, 32 * kRows, march_smem<S, MU>(), s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(share == 1, march_kernel<MODE, S, MU, REC>, (unsigned)blocks, 32 * kRows, march_smem<S, MU>(), s, a);
 }
 
 template <int MODE>

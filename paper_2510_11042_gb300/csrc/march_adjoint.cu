@@ -167,7 +167,9 @@ __global__ void __launch_bounds__(32 * kRows, 1) march_adjoint_kernel(const __gr
     const int xc = min(max(cx.x, 0), a.nxp - 2);
     const int y0 = chunk * a.rows, y1 = min(a.ny, y0 + a.rows);
     const int pa = max(y0 - (K - 1), 0), pend = min(y1 - 1 + (K - 1), a.ny - 1);
+    chain_release();
     init_rows(done);
+    chain_wait();
     unsigned char *stage = smem + Y::BYTES + w * G::BYTES;
     int r = pa + w;
     if (r <= pend) stage_row<MODE>(a, smem_u32(stage), lane, r, xc);
@@ -282,8 +284,7 @@ template <int MODE> cudaError_t launch_t(MarchAdjointArgs a, cudaStream_t s)
     a.rows = march_rows(a.ny, a.strips, (long long)std::max(1, sm_count()) * bps);
     const long long blocks = (long long)((a.ny + a.rows - 1) / a.rows) * a.strips;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    march_adjoint_kernel<MODE><<<(unsigned)blocks, 32 * kRows, AdjStage<MODE>::SMEM, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(true, march_adjoint_kernel<MODE>, (unsigned)blocks, 32 * kRows, AdjStage<MODE>::SMEM, s, a);
 }
 
 }  // namespace

@@ -107,6 +107,8 @@ __global__ void __launch_bounds__(BX, (ANA && MODE == 2) ? 5 : 7) step_kernel_ce
 {
     constexpr int R = ONE ? 1 : rows_of<S>();
     const int b = blockIdx.x;
+    chain_release();
+    chain_wait();
     if (a.line_on) {
         const int s = b * blockDim.x + threadIdx.x;
         if (s < a.n_line) line_work<MODE>(a, s);
@@ -325,15 +327,12 @@ cudaError_t launch_cell(StepArgs a, cudaStream_t s)
     if (ANA != (a.tfsf == 2)) return cudaErrorInvalidValue;
     if constexpr (MODE == 2 && !REC) {
         if (direct) {
-            step_kernel_cell<MODE, S, kBX, REC, MU, ANA, true, kDirect><<<a.nblk_main, tx, 0, s>>>(a);
-            return cudaGetLastError();
+            return launch_chained(a.chain != 0, step_kernel_cell<MODE, S, kBX, REC, MU, ANA, true, kDirect>, a.nblk_main, tx, 0, s, a);
         }
     }
     if (a.rows_per_block == 1)
-        step_kernel_cell<MODE, S, kBX, REC, MU, ANA, true><<<a.nblk_main, tx, 0, s>>>(a);
-    else
-        step_kernel_cell<MODE, S, kBX, REC, MU, ANA, false><<<a.nblk_main, tx, 0, s>>>(a);
-    return cudaGetLastError();
+        return launch_chained(a.chain != 0, step_kernel_cell<MODE, S, kBX, REC, MU, ANA, true>, a.nblk_main, tx, 0, s, a);
+    return launch_chained(a.chain != 0, step_kernel_cell<MODE, S, kBX, REC, MU, ANA, false>, a.nblk_main, tx, 0, s, a);
 }
 
 template <int MODE, class S>
