@@ -382,7 +382,9 @@ static cudaError_t probe_t(const void *f, float sc, long long P, int ny, int nxp
 // population fetched every sector of a group two or four times, which with
 // 64-bit divides held the old kernels at a tenth of the copy bandwidth), each
 // population scaled and completed by its incident part before it is summed in
-// direction order.  The closed-form wave is evaluated once per cell.
+// direction order.  All populations are loaded before any incident part: with
+// the two alternating per direction a cell took a load's latency seven times.
+// The closed-form wave is evaluated once per cell.
 template <int MODE, class S>
 __device__ __forceinline__ void cell_DB(const S *f, float sc, long long P, int c, const IncView &inc, int x, int y,
                                         int z, float D[3], float B[3])
@@ -390,44 +392,57 @@ __device__ __forceinline__ void cell_DB(const S *f, float sc, long long P, int c
     using PL = Planes<MODE>;
     using M = Mode<MODE>;
     constexpr int NC = PL::NC, NE = PL::NE;
+    float v[7 * NC];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+        const S *g = f + (long long)i * NC * P;
+        float *w = v + i * NC;
+        if constexpr (NC == 3) {
+            Io<S>::ld2(g, c, w[0], w[1]);
+            Io<S>::ld1(g + 2 * P, c, w[2]);
+        } else if constexpr (sizeof(S) == 4) {
+            Io<S>::ld2(g, c, w[0], w[1]);
+            Io<S>::ld2(g + 2 * P, c, w[2], w[3]);
+            Io<S>::ld2(g + 4 * P, c, w[4], w[5]);
+        } else {
+            Io<S>::ld4(g, c, w[0], w[1], w[2], w[3]);
+            Io<S>::ld2(g + 4 * P, c, w[4], w[5]);
+        }
+    }
     const bool in = inc.on && in_box(x, y, z, inc.tf_lo, inc.tf_hi);
-    float E0[3] = {0.f, 0.f, 0.f}, H0[3] = {0.f, 0.f, 0.f};
-    if (in && inc.on == 2) {
+    if (in && inc.on == 1) {
+        const float *l = inc.line + (inc.axis == 0 ? x : (inc.axis == 1 ? y : z));
+        float add[7 * NC];
+#pragma unroll
+        for (int k = 0; k < 7 * NC; ++k) add[k] = __ldg(l + (size_t)slot_plane(MODE, k / NC, k % NC) * inc.n);
+#pragma unroll
+        for (int k = 0; k < 7 * NC; ++k) v[k] = v[k] * sc + add[k];
+    } else if (in) {
         const float amp = (float)pw_amplitude(inc.pw, x, y, z, inc.t);
+        float E0[3], H0[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             E0[k] = amp * (float)inc.pw.pol[k];
             H0[k] = amp * (float)inc.pw.kxp[k];
         }
+#pragma unroll
+        for (int k = 0; k < 7 * NC; ++k) {
+            const int i = k / NC, s = k % NC, a = s < NE ? M::ec(s) : M::hc(s - NE);
+            const float add = i == 0 ? 0.f
+                                     : (s < NE ? E0[a] - cross_c(i, H0, a) : H0[a] + cross_c(i, E0, a)) * (1.0f / 6.0f);
+            v[k] = v[k] * sc + add;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 7 * NC; ++k) v[k] *= sc;
     }
-    const int sl = inc.axis == 0 ? x : (inc.axis == 1 ? y : z);
     D[0] = D[1] = D[2] = 0.f;
     B[0] = B[1] = B[2] = 0.f;
 #pragma unroll
-    for (int i = 0; i < 7; ++i) {
-        const S *g = f + (long long)i * NC * P;
-        float v[NC];
-        if constexpr (NC == 3) {
-            Io<S>::ld2(g, c, v[0], v[1]);
-            Io<S>::ld1(g + 2 * P, c, v[2]);
-        } else if constexpr (sizeof(S) == 4) {
-            Io<S>::ld2(g, c, v[0], v[1]);
-            Io<S>::ld2(g + 2 * P, c, v[2], v[3]);
-            Io<S>::ld2(g + 4 * P, c, v[4], v[5]);
-        } else {
-            Io<S>::ld4(g, c, v[0], v[1], v[2], v[3]);
-            Io<S>::ld2(g + 4 * P, c, v[4], v[5]);
-        }
-#pragma unroll
-        for (int s = 0; s < NC; ++s) {
-            const int a = s < NE ? M::ec(s) : M::hc(s - NE);
-            float add = 0.f;
-            if (in) {
-                if (inc.on == 1) add = __ldg(inc.line + (size_t)slot_plane(MODE, i, s) * inc.n + sl);
-                else if (i) add = (s < NE ? E0[a] - cross_c(i, H0, a) : H0[a] + cross_c(i, E0, a)) * (1.0f / 6.0f);
-            }
-            (s < NE ? D : B)[a] += v[s] * sc + add;
-        }
+    for (int k = 0; k < 7 * NC; ++k) {
+        const int s = k % NC;
+        if (s < NE) D[M::ec(s)] += v[k];
+        else B[M::hc(s - NE)] += v[k];
     }
 }
 
@@ -436,7 +451,7 @@ constexpr int kEThreads = 256;
 // E and H maps in one pass over the populations (components 0..2: E, 3..5: H;
 // a null pointer is skipped).  Bound by HBM: the populations and 1/eps_r once,
 // 4 B a component out.  One launch a component read the populations six times:
-// 384^3 FP32 59.9 -> 2.36 ms, FP16 57.4 -> 2.36, 1024^2 EZ 0.575 -> 0.067.
+// 384^3 FP32 59.9 -> 1.59 ms, FP16 57.4 -> 1.31, 1024^2 EZ 0.575 -> 0.047.
 struct FieldOut { float *p[6]; };
 template <int MODE, class S>
 __global__ void __launch_bounds__(kEThreads) fields_kernel(const S *f, const float *inv_eps, const float *inv_mu,
@@ -461,7 +476,7 @@ __global__ void __launch_bounds__(kEThreads) fields_kernel(const S *f, const flo
 
 // Field energy 1/2 sum (|D|^2 / eps + |B|^2 / mu), FP64 per block; HBM and the
 // FP64 pipe (about 15 operations a cell) take about the same time in FP32
-// storage.  384^3 FP32 15.8 -> 3.15 ms, 1024^2 EZ 0.355 -> 0.088.
+// storage.  384^3 FP32 15.8 -> 1.84 ms, FP16 14.3 -> 1.84, 1024^2 EZ 0.355 -> 0.073.
 template <int MODE, class S>
 __global__ void __launch_bounds__(kEThreads) energy_partial(const S *f, const float *inv_eps, const float *inv_mu,
                                                             float sc, long long P, int nx, int ny, int nxp,
