@@ -184,8 +184,9 @@ __global__ void __launch_bounds__(BX, (aa_blocks<MODE, S, ANA>())) aa_step_kerne
         const int s = b * blockDim.x + threadIdx.x;
         if (s < a.n_line) line_work<MODE>(a, s);
     }
-    const int r = b / a.nblk_x;
-    aa_row<MODE, S, BX, MU, ANA, KIND, FORM>(a, g, b % a.nblk_x, r % a.ny, r / a.ny);
+    const int tile = a.flip ? a.nblk_main - 1 - b : b;
+    const int r = tile / a.nblk_x;
+    aa_row<MODE, S, BX, MU, ANA, KIND, FORM>(a, g, tile % a.nblk_x, r % a.ny, r / a.ny);
 }
 
 // The face cell k of axis ax (the other two coordinates, the lower one

@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kAdjBX, MODE == 2 ? 7 : 1) adjoint_step_kernel
     using PL = Planes<MODE>;
     using M = Mode<MODE>;
     constexpr int Q = PL::Q;
-    const int b = blockIdx.x;
+    const int b = a.flip ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
     chain_release();
     chain_wait();
     const int bx = b % a.nblk_x;

@@ -882,6 +882,7 @@ static void step_args_at(lbem_ctx *h, StepArgs &a, int64_t tn, int in, int out)
         a.fin_q[q] = (const char *)h->f[in] + q * plane_bytes;
         a.fout_q[q] = (char *)h->f[out] + q * plane_bytes;
     }
+    a.flip = (int)(tn & 1);
     a.dft_on = 0;
     if (h->has_wave) {
         if (!h->analytic) {
@@ -2334,6 +2335,7 @@ int32_t lbem_adjoint(lbem_handle h, const double *theta, const double *phi, cons
                 a.line_out = rl.at(t + 2);
                 source_fields(h, t + 2, a.src_E, a.src_H);
                 a.rec = rec + (size_t)k * NE * h->P;
+                a.flip = (int)(k & 1);
                 const cudaError_t e = launch_step_record(h->g.mode, a, h->stream);
                 if (e != cudaSuccess) return cuda_fail(h, e, "replay step launch");
                 k += 1;
@@ -2373,6 +2375,7 @@ int32_t lbem_adjoint(lbem_handle h, const double *theta, const double *phi, cons
                     b.lout_q[q] = mu[mcur ^ 1] + (size_t)q * h->P;
                 }
                 b.rec = rec + (size_t)k * NE * h->P;
+                b.flip = (int)(k & 1);
                 b.dft_on = phase_at(t0 + k + 1, b.dft_c, b.dft_s);
                 e = launch_adjoint_step(h->g.mode, b, h->stream);
                 k -= 1;

@@ -273,6 +273,16 @@ struct StepArgs {
     // reduced-precision storage: stored = population / scale (power of two)
     float scale, inv_scale;
     int chain;                 // launch chained to the kernel before it (launch_chained)
+    // Tiles from the last to the first, on every other step: a step then starts
+    // on the cells the one before it wrote last, which L2 (129 MB) still holds,
+    // where the same order each time finds only evicted lines.  us a single step,
+    // same order -> alternating: 96^3 FP32 46.1 -> 41.5, in place 46.9 -> 36.0;
+    // 2048^2 EZ FP16 71.4 -> 63.4; 4000^2 EZ FP32 410 -> 391; 300^3 BF16 in place
+    // 756 -> 746; 96^3 adjoint replay 48.1 -> 43.9, backward 52.1 -> 47.2.  Passes
+    // of several steps keep one order: fewer bytes return through L2 there and
+    // the index arithmetic costs the 16-bit kernels (300^3 FP16 429 -> 434,
+    // 4000^2 EZ FP16 127.0 -> 128.5; FP32 470 -> 471 at 256^3).
+    int flip;
     // forward replay for the adjoint: total-field D of the pulled populations
     // (scattered D plus the incident D inside the total-field box), NE planes
     // of P floats, written only by the recording kernel
@@ -526,6 +536,7 @@ struct AdjointArgs {
     int nx, ny, nz, nxp;
     long long P;
     int nblk_x;
+    int flip;                  // as StepArgs::flip
     int w;
     float sigma_max, inv_w;
     // sensitivity of J to the DFT samples of step t (fields at time t)

@@ -113,8 +113,9 @@ __global__ void __launch_bounds__(BX, (ANA && MODE == 2) ? 5 : 7) step_kernel_ce
         const int s = b * blockDim.x + threadIdx.x;
         if (s < a.n_line) line_work<MODE>(a, s);
     }
-    const int bx = b % a.nblk_x;
-    const int r0 = (b / a.nblk_x) * R;
+    const int tile = a.flip ? a.nblk_main - 1 - b : b;
+    const int bx = tile % a.nblk_x;
+    const int r0 = (tile / a.nblk_x) * R;
     const int r1 = min(r0 + R, a.ny * a.nz);
     for (int r = r0; r < r1; ++r) row_cells<MODE, S, BX, REC, MU, ANA, FORM>(a, bx, r % a.ny, r / a.ny);
 }
