@@ -920,7 +920,6 @@ static void stage_slot(lbem_ctx *h, StepArgs &a)
     if (!a.dft_on || h->xs_n == 0) return;
     a.xstage = h->xstage + ((size_t)h->xs_bank * kXBank + h->xs_cnt) * h->NC * h->xs_n;
     a.xs_n = h->xs_n;
-    for (int f = 0; f < h->faces.nfaces; ++f) a.xs_start[f] = h->faces.cell_start[f];
     h->xs_sc[h->xs_cnt] = a.dft_sc;
     h->xs_ss[h->xs_cnt] = a.dft_ss;
     ++h->xs_cnt;

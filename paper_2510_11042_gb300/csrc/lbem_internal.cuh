@@ -256,7 +256,6 @@ struct StepArgs {
     double dft_sc, dft_ss;     // dft_scale_cells times cos, sin of the step's phase
     float *xstage;             // 3D, non-NULL: staged face fields go here ([NC][xs_n]) for dft_flush_x
     long long xs_n;            // cells of all faces (one component of one staged step)
-    long long xs_start[kMaxFaces];  // first staged cell of each face
     // 3D: the box planes of each axis with faces (-1 for a 1-cell axis, which
     // has none), and the first staged cell of each face
     int ft_lo[3], ft_hi[3], ft_at[3][2];
@@ -488,6 +487,7 @@ struct FarFieldArgs {
     float2 *x32;               // packed face phasors [face][nup][4][nvp], weights folded in
     float2 *tab32;             // phase tables [n0 + n1 + n2][n_ang_pad]
     long long x32_cap, tab32_cap;  // capacities in float2
+    int fine_log2;             // far_field_columns: offsets per coarse phase entry (set by the launcher)
     int n_ang_pad;             // n_ang rounded up to the angle tile
     int uc;                    // face rows per chunk
     int nup[kMaxFaces], nvp[kMaxFaces];  // padded rows / columns per face

@@ -35,21 +35,49 @@ __device__ __forceinline__ double warp_sum(double v)
 
 // ------------------------------------------------------------ far field
 constexpr int kFFThreads = 256;
-constexpr int kFFFine = 64;         // coordinates per coarse phase entry
 constexpr int kFFTableMax = 4480;   // phase entries held in shared memory (70 KB)
 
 // How a block of far_field_columns gets its phases exp(j k r_a (p_a - c_a)):
-// evaluated at each use; as products of a coarse entry (every 64th coordinate)
-// and a fine one (the 64 offsets), tabulated per block; or from a table of
-// every coordinate of the box, filled with those products.
+// evaluated at each use; as products of a coarse entry (every F-th coordinate)
+// and a fine one (the F offsets), tabulated per block; or from a table of
+// every coordinate of the box, filled with those products.  F = 2^fine_log2 gives
+// the fewest entries.
 enum FFPhase { FF_DIRECT = 0, FF_FACTORED = 1, FF_TABLE = 2 };
 
-__host__ __device__ inline int ff_coarse(int n) { return (n + kFFFine - 1) / kFFFine; }
-inline int ff_factored_entries(const FaceGeom &g)
+__host__ __device__ inline int ff_entries(int n, int lg) { return (1 << lg) + ((n + (1 << lg) - 1) >> lg); }
+inline int ff_factored_entries(int mode, const FaceGeom &g, int lg)
 {
     int e = 0;
-    for (int ax = 0; ax < 3; ++ax) e += kFFFine + ff_coarse(g.hi[ax] - g.lo[ax] + 1);
+    for (int ax = 0; ax < (mode == 2 ? 3 : 2); ++ax) e += ff_entries(g.hi[ax] - g.lo[ax] + 1, lg);
     return e;
+}
+
+// The outputs a mode has among N_xyz, L_xyz (Re, Im): EZ N_z, L_x, L_y; HZ N_x,
+// N_y, L_z; 3D all twelve.  Output i of a mode's list, and an output's place.
+template <int MODE> __host__ __device__ constexpr int ff_outs() { return MODE == 2 ? 12 : 6; }
+template <int MODE> __host__ __device__ constexpr int ff_out(int i)
+{
+    return MODE == 2 ? i : (MODE == 0 ? 4 + i : (i < 4 ? i : 6 + i));
+}
+
+// Reduce-scatter of N = 8 or 16 values over the warp: each step a lane keeps the
+// half of its values that its bit H selects and adds its partner's copy of that
+// half; the steps that are left sum the one value.  Lane l then holds the warp's
+// sum of value l / (32 / N).
+template <int N> __device__ __forceinline__ double warp_scatter(double (&v)[N], int lane)
+{
+    int off = 16;
+#pragma unroll
+    for (int h = N / 2; h >= 1; h /= 2, off /= 2) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int j = 0; j < h; ++j) {
+            const double send = up ? v[j] : v[j + h];
+            v[j] = (up ? v[j + h] : v[j]) + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+    }
+    for (; off >= 1; off /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+    return v[0];
 }
 
 // Stage 1: one block per (chunk of face columns, angle); writes 12 doubles
@@ -60,36 +88,45 @@ inline int ff_factored_entries(const FaceGeom &g)
 // alone; the column factor t_v(iv) w(iv) t_w multiplies the four column sums
 // once, and J = n x H, M = -n x E are formed from them.  Per (cell, angle) this
 // is four complex multiply-adds.  Bound by the FP64 pipe (two operations a
-// clock per SM), so what counts in 2D, where a column is one cell, is the
-// number of FP64 sincos: a table of every coordinate per block cost 16 blocks x
-// 1970 of them an angle on a 1024^2 grid (0.60 ms for 181 angles); factored and
-// with few blocks an angle the call takes 0.133 ms.  A 4000^2 box, too long
-// for that table, evaluated the phase of every (cell, angle): 0.97 -> 0.228 ms.
+// clock per SM), so what counts in 2D, where a column is one cell, is the FP64
+// work beside the columns: the sincos of the phase entries, and the reduction
+// over the block.  A table of every coordinate per block cost 16 blocks x 1970
+// sincos an angle on a 1024^2 grid (0.60 ms for 181 angles); factored and with few
+// blocks an angle the call took 0.127 ms; with the direction found by one warp,
+// the faces' own factors kept, the fewest entries and a reduce-scatter of the
+// mode's outputs alone it takes 0.100 (520^2 HZ: the kernel 48 -> 27 us, the call
+// 92 -> 62).  A 4000^2 box, too long for that table, evaluated the phase of every
+// (cell, angle): 0.97 -> 0.228 -> 0.182 ms.
 template <int MODE, int PH>
 __global__ void __launch_bounds__(kFFThreads) far_field_columns(const FarFieldArgs a)
 {
     extern __shared__ double2 ff_tab[];
+    constexpr int AXES = MODE == 2 ? 3 : 2;
+    chain_release();
     const int ang = blockIdx.y;
-    const double th = a.theta[ang];
-    double rh[3];
-    if (MODE == 2) {
-        const double ph = a.phi[ang];
-        rh[0] = sin(th) * cos(ph);
-        rh[1] = sin(th) * sin(ph);
-        rh[2] = cos(th);
-    } else {
-        rh[0] = cos(th);
-        rh[1] = sin(th);
-        rh[2] = 0.0;
+    // the direction, by one warp (odd lanes take phi)
+    __shared__ double rh[3];
+    if (threadIdx.x < 32) {
+        const bool odd = MODE == 2 && (threadIdx.x & 1);
+        double sn, cs;
+        sincos(odd ? a.phi[ang] : a.theta[ang], &sn, &cs);
+        const double sp = __shfl_sync(0xffffffffu, sn, 1), cp = __shfl_sync(0xffffffffu, cs, 1);
+        if (threadIdx.x == 0) {
+            rh[0] = MODE == 2 ? sn * cp : cs;
+            rh[1] = MODE == 2 ? sn * sp : sn;
+            rh[2] = MODE == 2 ? cs : 0.0;
+        }
     }
+    __syncthreads();
     const int n3[3] = {a.g.hi[0] - a.g.lo[0] + 1, a.g.hi[1] - a.g.lo[1] + 1, a.g.hi[2] - a.g.lo[2] + 1};
-    // factored entries of axis ax: the 64 fine ones at foff, then the coarse ones
-    const int foff[3] = {0, kFFFine + ff_coarse(n3[0]), 2 * kFFFine + ff_coarse(n3[0]) + ff_coarse(n3[1])};
-    const int nfac = foff[2] + kFFFine + ff_coarse(n3[2]);
+    // factored entries of axis ax: the F fine ones at foff, then the coarse ones
+    const int lg = a.fine_log2, fine = 1 << lg;
+    const int foff[3] = {0, ff_entries(n3[0], lg), ff_entries(n3[0], lg) + ff_entries(n3[1], lg)};
+    const int nfac = foff[2] + (AXES == 3 ? ff_entries(n3[2], lg) : 0);
     const int toff[3] = {nfac, nfac + n3[0], nfac + n3[0] + n3[1]};
     auto cmul = [](double2 p, double2 q) { return make_double2(p.x * q.x - p.y * q.y, p.x * q.y + p.y * q.x); };
     auto factored = [&](int ax, int e) {
-        return cmul(ff_tab[foff[ax] + kFFFine + e / kFFFine], ff_tab[foff[ax] + e % kFFFine]);
+        return cmul(ff_tab[foff[ax] + fine + (e >> lg)], ff_tab[foff[ax] + (e & (fine - 1))]);
     };
     auto phase = [&](int ax, int e) {
         if constexpr (PH == FF_TABLE) return ff_tab[toff[ax] + e];
@@ -100,9 +137,9 @@ __global__ void __launch_bounds__(kFFThreads) far_field_columns(const FarFieldAr
     };
     if constexpr (PH != FF_DIRECT) {
         for (int e = threadIdx.x; e < nfac; e += blockDim.x) {
-            const int ax = e < foff[1] ? 0 : (e < foff[2] ? 1 : 2);
+            const int ax = e < foff[1] ? 0 : (AXES == 2 || e < foff[2] ? 1 : 2);
             const int i = e - foff[ax];
-            const double pos = i < kFFFine ? (double)i : a.g.lo[ax] + (double)(i - kFFFine) * kFFFine - a.center[ax];
+            const double pos = i < fine ? (double)i : a.g.lo[ax] + (double)(i - fine) * fine - a.center[ax];
             double sp, cp;
             sincos(a.k * rh[ax] * pos, &sp, &cp);
             ff_tab[e] = make_double2(cp, sp);
@@ -116,6 +153,15 @@ __global__ void __launch_bounds__(kFFThreads) far_field_columns(const FarFieldAr
         }
         __syncthreads();
     }
+    // the faces' own factors t_w, times the outward normal's sign
+    __shared__ double2 tw[kMaxFaces];
+    if (threadIdx.x < a.g.nfaces) {
+        const int f = threadIdx.x, ax = a.g.axis[f];
+        double2 p = phase(ax, a.g.side[f] ? n3[ax] - 1 : 0);
+        if (!a.g.side[f]) p = make_double2(-p.x, -p.y);
+        tw[f] = p;
+    }
+    __syncthreads();
 
     int ncols = 0;
     for (int f = 0; f < a.g.nfaces; ++f) ncols += a.g.nv[f];
@@ -157,11 +203,12 @@ __global__ void __launch_bounds__(kFFThreads) far_field_columns(const FarFieldAr
                 }
             }
         }
-        // column factor t_v(iv) w_v(iv) t_w and the outward normal's sign
-        double2 cf = cmul(phase(va, iv), phase(ax, a.g.side[f] ? n3[ax] - 1 : 0));
-        const double w = (nv > 1 && (iv == 0 || iv == nv - 1) ? 0.5 : 1.0) * (a.g.side[f] ? 1.0 : -1.0);
-        cf.x *= w;
-        cf.y *= w;
+        // column factor t_v(iv) w_v(iv) t_w
+        double2 cf = cmul(phase(va, iv), tw[f]);
+        if (nv > 1 && (iv == 0 || iv == nv - 1)) {
+            cf.x *= 0.5;
+            cf.y *= 0.5;
+        }
         // J_b1 = -sgn H_b2, J_b2 = sgn H_b1, M_b1 = sgn E_b2, M_b2 = -sgn E_b1
         auto add = [&](int m, double s, double xr, double xi) {
             acc[m] = fma(s * cf.x, xr, fma(-s * cf.y, xi, acc[m]));
@@ -181,48 +228,69 @@ __global__ void __launch_bounds__(kFFThreads) far_field_columns(const FarFieldAr
         else if (MODE == 2) column(std::integral_constant<int, 2>(), f, iv);
     }
 
-    __shared__ double red[kFFThreads / 32][12];
+    constexpr int NO = ff_outs<MODE>(), N = MODE == 2 ? 16 : 8;
+    __shared__ double red[kFFThreads / 32][N];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    double v[N];
 #pragma unroll
-    for (int m = 0; m < 12; ++m) {
-        const double v = warp_sum(acc[m]);
-        if (lane == 0) red[wid][m] = v;
-    }
+    for (int i = 0; i < N; ++i) v[i] = i < NO ? acc[ff_out<MODE>(i < NO ? i : 0)] : 0.0;
+    const double sum = warp_scatter(v, lane);
+    if (lane % (32 / N) == 0) red[wid][lane / (32 / N)] = sum;
     __syncthreads();
     if (threadIdx.x < 12) {
         double s = 0.0;
-        for (int wi = 0; wi < kFFThreads / 32; ++wi) s += red[wi][threadIdx.x];
+#pragma unroll
+        for (int i = 0; i < NO; ++i)
+            if (ff_out<MODE>(i) == threadIdx.x)
+                for (int wi = 0; wi < kFFThreads / 32; ++wi) s += red[wi][i];
         a.partial[((long long)ang * a.chunks + blockIdx.x) * 12 + threadIdx.x] = s;
     }
 }
 
-// Stage 2: one thread per angle; fixed-order sum over chunks, then Eq. 5/6.
-__global__ void far_field_finalize(const FarFieldArgs a)
+// Stage 2: fixed-order sum over chunks, then Eq. 5/6.  Twelve threads an angle
+// sum one output each, then one lane an angle goes on.  FP64 again: a warp's
+// instruction holds the pipe for 16 clocks however many lanes it has, so the
+// angles are spread over the SMs and no lane repeats another's work (181 angles
+// alone and cold: 10.4 us with 128 angles a block, 8.1 with eight).  What does not
+// need the sums runs before the wait for them, beside the kernel that makes them.
+constexpr int kFinAngles = 8;
+__global__ void __launch_bounds__(12 * kFinAngles) far_field_finalize(const FarFieldArgs a)
 {
-    const int ang = blockIdx.x * blockDim.x + threadIdx.x;
-    if (ang >= a.n_ang) return;
-    double v[12];
-    for (int m = 0; m < 12; ++m) v[m] = 0.0;
-    for (int c = 0; c < a.chunks; ++c)
-        for (int m = 0; m < 12; ++m) v[m] += a.partial[((long long)ang * a.chunks + c) * 12 + m];
-    // |E_I|: incident-line E phasor along pol, mean over the two nodes around the centre
-    double ei = 0.0;
-    const int nodes[2] = {a.center_i0, a.center_i1};
-    for (int t = 0; t < 2 && a.ei_fixed <= 0.0; ++t) {
-        double re = 0.0, im = 0.0;
-        for (int c = 0; c < 3; ++c) {
-            re += a.pol[c] * a.line_dft[(nodes[t] * 3 + c) * 2 + 0];
-            im += a.pol[c] * a.line_dft[(nodes[t] * 3 + c) * 2 + 1];
+    __shared__ double sums[kFinAngles * 12];
+    const int ang0 = blockIdx.x * kFinAngles, ang = ang0 + threadIdx.x;
+    const bool mine = threadIdx.x < kFinAngles && ang < a.n_ang;
+    double ei = 0.0, st = 0.0, ct = 1.0, sp = 0.0, cp = 1.0;
+    if (mine) {
+        // |E_I|: incident-line E phasor along pol, mean over the two nodes around the centre
+        const int nodes[2] = {a.center_i0, a.center_i1};
+        for (int t = 0; t < 2 && a.ei_fixed <= 0.0; ++t) {
+            double re = 0.0, im = 0.0;
+            for (int c = 0; c < 3; ++c) {
+                re += a.pol[c] * a.line_dft[(nodes[t] * 3 + c) * 2 + 0];
+                im += a.pol[c] * a.line_dft[(nodes[t] * 3 + c) * 2 + 1];
+            }
+            ei += 0.5 * sqrt(re * re + im * im);
         }
-        ei += 0.5 * sqrt(re * re + im * im);
+        if (a.ei_fixed > 0.0) ei = a.ei_fixed;
+        sincos(a.theta[ang], &st, &ct);
+        if (a.mode == 2) sincos(a.phi[ang], &sp, &cp);
     }
-    if (a.ei_fixed > 0.0) ei = a.ei_fixed;
-    const double th = a.theta[ang];
+    chain_wait();
+    const int j = threadIdx.x / 12, m0 = threadIdx.x % 12;
+    if (ang0 + j < a.n_ang) {
+        const double *p = a.partial + (long long)(ang0 + j) * a.chunks * 12 + m0;
+        double sum = 0.0;
+#pragma unroll 8
+        for (int c = 0; c < a.chunks; ++c) sum += p[c * 12];
+        sums[threadIdx.x] = sum;
+        if (a.amp) a.amp[(long long)ang0 * 12 + threadIdx.x] = sum;
+    }
+    __syncthreads();
+    if (!mine) return;
+    const double *v = sums + 12 * threadIdx.x;
     const double k = a.k;
     double s2;
     if (a.mode == 2) {
-        const double ph = a.phi[ang];
-        const double st = sin(th), ct = cos(th), sp = sin(ph), cp = cos(ph);
         const double tv[3] = {ct * cp, ct * sp, -st}, pv[3] = {-sp, cp, 0.0};
         double Nt[2] = {0, 0}, Np[2] = {0, 0}, Lt[2] = {0, 0}, Lp[2] = {0, 0};
         for (int c = 0; c < 3; ++c)
@@ -237,7 +305,7 @@ __global__ void far_field_finalize(const FarFieldArgs a)
         s2 = k * k * k * k * (a1r * a1r + a1i * a1i + a2r * a2r + a2i * a2i) /
              (16.0 * M_PI * M_PI * ei * ei);
     } else {
-        const double pv[3] = {-sin(th), cos(th), 0.0};
+        const double pv[3] = {-st, ct, 0.0};
         double Np[2] = {0, 0}, Lp[2] = {0, 0};
         for (int c = 0; c < 3; ++c)
             for (int r = 0; r < 2; ++r) {
@@ -250,8 +318,6 @@ __global__ void far_field_finalize(const FarFieldArgs a)
         s2 = k * k * (ar * ar + ai * ai) / (8.0 * M_PI * ei * ei);
     }
     a.s2[ang] = s2;
-    if (a.amp)
-        for (int m = 0; m < 12; ++m) a.amp[(long long)ang * 12 + m] = v[m];
 }
 
 // ------------------------------------------------------------ permittivity
@@ -559,39 +625,78 @@ constexpr int kF32Rows = 16;     // face rows staged in shared memory per pass
 
 // Phase tables tab32[e][a] = exp(j k r_ax(a) (p_e - c_ax)) for the box
 // coordinates p_e along x, y, z (e in [0, n0 + n1 + n2)); zero for padded angles.
-__global__ void ff32_tables(const FarFieldArgs a)
+// A block fills 32 angles x 32 coordinates of one axis with products of 4 coarse
+// and 8 fine phases an angle, formed from two phases by multiplication: FP64-bound,
+// and a sincos and the direction's own sines per entry were ten times the work
+// (the whole call, 543 angles: 384^3 0.600 -> 0.504 ms, 64^3 0.113 -> 0.088).
+constexpr int kTabCoords = 32, kTabFine = 8;
+__device__ __forceinline__ void ff32_tables(const FarFieldArgs &a, int block)
 {
-    const int n0 = a.g.hi[0] - a.g.lo[0] + 1, n1 = a.g.hi[1] - a.g.lo[1] + 1,
-              n2 = a.g.hi[2] - a.g.lo[2] + 1;
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)(n0 + n1 + n2) * a.n_ang_pad) return;
-    const int ang = (int)(i % a.n_ang_pad), e = (int)(i / a.n_ang_pad);
-    float2 out = make_float2(0.f, 0.f);
-    if (ang < a.n_ang) {
-        const int ax = e < n0 ? 0 : (e < n0 + n1 ? 1 : 2);
-        const int toff = ax == 0 ? 0 : (ax == 1 ? n0 : n0 + n1);
-        const double th = a.theta[ang], ph = a.phi[ang];
-        const double r = ax == 0 ? sin(th) * cos(ph) : (ax == 1 ? sin(th) * sin(ph) : cos(th));
-        const double pos = a.g.lo[ax] + (e - toff);
-        double sp, cp;
-        sincos(a.k * r * (pos - a.center[ax]), &sp, &cp);
-        out = make_float2((float)cp, (float)sp);
+    __shared__ double2 fine[kTabFine + 1][32], coarse[kTabCoords / kTabFine][32];
+    const int tiles = a.n_ang_pad / 32;
+    const int ang0 = block % tiles * 32;
+    int ax = 0, e0 = block / tiles * kTabCoords, toff = 0, n = a.g.hi[0] - a.g.lo[0] + 1;
+    while (e0 >= n) {
+        e0 -= (n + kTabCoords - 1) / kTabCoords * kTabCoords;
+        toff += n;
+        ++ax;
+        n = a.g.hi[ax] - a.g.lo[ax] + 1;
     }
-    a.tab32[i] = out;
+    auto cmul = [](double2 p, double2 q) { return make_double2(p.x * q.x - p.y * q.y, p.x * q.y + p.y * q.x); };
+    const int j = threadIdx.x % 32, wid = threadIdx.x / 32, ang = ang0 + j;
+    double2 first = make_double2(1.0, 0.0);
+    if (wid < 2 && ang < a.n_ang) {   // the phase of one cell, and of the block's first coordinate
+        const double th = a.theta[ang];
+        const double r = ax == 2 ? cos(th) : sin(th) * (ax == 0 ? cos(a.phi[ang]) : sin(a.phi[ang]));
+        sincos(a.k * r * (wid == 0 ? 1.0 : a.g.lo[ax] + (double)e0 - a.center[ax]), &first.y, &first.x);
+    }
+    if (wid == 0) {
+        const double2 p2 = cmul(first, first), p4 = cmul(p2, p2);
+        fine[0][j] = make_double2(1.0, 0.0);
+        fine[1][j] = first;
+        fine[2][j] = p2;
+        fine[3][j] = cmul(p2, first);
+        fine[4][j] = p4;
+        fine[5][j] = cmul(p4, first);
+        fine[6][j] = cmul(p4, p2);
+        fine[7][j] = cmul(p4, cmul(p2, first));
+        fine[8][j] = cmul(p4, p4);
+    }
+    __syncthreads();
+    if (wid == 1) {
+        const double2 p8 = fine[8][j], p16 = cmul(p8, p8);
+        coarse[0][j] = first;
+        coarse[1][j] = cmul(first, p8);
+        coarse[2][j] = cmul(first, p16);
+        coarse[3][j] = cmul(first, cmul(p16, p8));
+    }
+    __syncthreads();
+    for (int i = wid; i < min(kTabCoords, n - e0); i += kF32Threads / 32) {
+        const double2 p = cmul(coarse[i / kTabFine][j], fine[i % kTabFine][j]);
+        a.tab32[(long long)(toff + e0 + i) * a.n_ang_pad + ang] =
+            ang < a.n_ang ? make_float2((float)p.x, (float)p.y) : make_float2(0.f, 0.f);
+    }
 }
 
 // Packed faces x32[f][u][q][v] = w_u w_v X_q(u, v) in FP32, q = H_b1, H_b2,
 // E_b1, E_b2 (b1 = AX+1, b2 = AX+2 mod 3); zero in the padding.
-__global__ void ff32_pack(const FarFieldArgs a)
+__device__ __forceinline__ void ff32_pack(const FarFieldArgs &a, int block)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long i = (long long)block * kF32Threads + threadIdx.x;
     if (i >= a.off32[a.g.nfaces]) return;
     int f = 0;
     while (i >= a.off32[f + 1]) ++f;
     const long long r = i - a.off32[f];
     const int nvp = a.nvp[f];
-    const int v = (int)(r % nvp);
-    const long long t = r / nvp;
+    int v;
+    long long t;
+    if (r < 0x7fffffffLL) {   // 32-bit division wherever it serves
+        v = (int)((unsigned)r % (unsigned)nvp);
+        t = (unsigned)r / (unsigned)nvp;
+    } else {
+        v = (int)(r % nvp);
+        t = r / nvp;
+    }
     const int q = (int)(t % 4), u = (int)(t / 4);
     const int nu = a.g.nu[f], nv = a.g.nv[f];
     float2 out = make_float2(0.f, 0.f);
@@ -606,6 +711,14 @@ __global__ void ff32_pack(const FarFieldArgs a)
         out = make_float2((float)(w * c[(2 * slot) * plane]), (float)(w * c[(2 * slot + 1) * plane]));
     }
     a.x32[i] = out;
+}
+
+// Both, in one launch: the first tab_blocks blocks take the tables.
+__global__ void __launch_bounds__(kF32Threads) ff32_prepare(const FarFieldArgs a, int tab_blocks)
+{
+    chain_release();
+    if ((int)blockIdx.x < tab_blocks) ff32_tables(a, blockIdx.x);
+    else ff32_pack(a, blockIdx.x - tab_blocks);
 }
 
 __device__ __forceinline__ void cmac(float &sr, float &si, float2 p, float xr, float xi)
@@ -638,6 +751,8 @@ __device__ __forceinline__ void rs_stage(float (&o)[32], int lane)
 __global__ void __launch_bounds__(kF32Threads, 2) far_field_f32(const FarFieldArgs a)
 {
     extern __shared__ float4 ff_sm[];
+    chain_release();
+    chain_wait();
     float2 *At = reinterpret_cast<float2 *>(ff_sm);                  // [uc][32] row phases
     float4 *Xs = ff_sm + a.uc * (kF32Angles / 2);                    // [16 rows x 4 q][32] (2 columns)
     double *acc = reinterpret_cast<double *>(Xs + kF32Rows * 4 * 32);  // [32 angles][12]
@@ -742,6 +857,11 @@ __global__ void __launch_bounds__(kF32Threads, 2) far_field_f32(const FarFieldAr
 
 }  // namespace
 
+static cudaError_t launch_finalize(const FarFieldArgs &a, cudaStream_t s)
+{
+    return launch_chained(true, far_field_finalize, (a.n_ang + kFinAngles - 1) / kFinAngles, 12 * kFinAngles, 0, s, a);
+}
+
 static size_t ff32_smem(int uc)
 {
     return (size_t)uc * kF32Angles * sizeof(float2) + (size_t)kF32Rows * 4 * 32 * sizeof(float4) +
@@ -814,13 +934,17 @@ static cudaError_t launch_far_field_f32(FarFieldArgs a, cudaStream_t s, int *lau
     for (int f = 0; f < a.g.nfaces; ++f) a.chunk_start[f + 1] = a.chunk_start[f] + (a.nup[f] + a.uc - 1) / a.uc;
     a.chunks = a.chunk_start[a.g.nfaces];
     const size_t sm = ff32_smem(a.uc);
-    const long long nt = (long long)ne * a.n_ang_pad;
-    ff32_tables<<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(a);
-    ff32_pack<<<(unsigned)((off + 255) / 256), 256, 0, s>>>(a);
-    far_field_f32<<<dim3(tiles, a.chunks), kF32Threads, sm, s>>>(a);
-    far_field_finalize<<<(a.n_ang + 127) / 128, 128, 0, s>>>(a);
-    if (launches) *launches += 4;
-    return cudaGetLastError();
+    long long tab_blocks = 0;
+    for (int ax = 0; ax < 3; ++ax) tab_blocks += (a.g.hi[ax] - a.g.lo[ax] + kTabCoords) / kTabCoords;
+    tab_blocks *= a.n_ang_pad / 32;
+    const long long blocks = tab_blocks + (off + kF32Threads - 1) / kF32Threads;
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+    ff32_prepare<<<(unsigned)blocks, kF32Threads, 0, s>>>(a, (int)tab_blocks);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = launch_chained(true, far_field_f32, dim3(tiles, a.chunks), kF32Threads, sm, s, a);
+    if (e == cudaSuccess) e = launch_finalize(a, s);
+    if (launches) *launches += 3;
+    return e;
 }
 
 // The FP64 projection's partial sums (the caller finalises).  In 3D a column
@@ -841,9 +965,12 @@ static cudaError_t far_field_columns_go(const FarFieldArgs &a, int entries, cuda
 }
 
 template <int MODE>
-static cudaError_t far_field_columns_t(const FarFieldArgs &a, cudaStream_t s)
+static cudaError_t far_field_columns_t(FarFieldArgs a, cudaStream_t s)
 {
-    const int fac = ff_factored_entries(a.g);
+    a.fine_log2 = 3;
+    for (int lg = 4; lg <= 8; ++lg)
+        if (ff_factored_entries(MODE, a.g, lg) < ff_factored_entries(MODE, a.g, a.fine_log2)) a.fine_log2 = lg;
+    const int fac = ff_factored_entries(MODE, a.g, a.fine_log2);
     if constexpr (MODE == 2) {
         int all = fac;
         for (int ax = 0; ax < 3; ++ax) all += a.g.hi[ax] - a.g.lo[ax] + 1;
@@ -881,9 +1008,8 @@ cudaError_t launch_far_field(const FarFieldArgs &a, cudaStream_t s, int *launche
     if (a.mode == 2 && a.x32 != nullptr) return launch_far_field_f32(a, s, launches);
     const cudaError_t e = launch_far_field_partial(a, s);
     if (e != cudaSuccess) return e;
-    far_field_finalize<<<(a.n_ang + 127) / 128, 128, 0, s>>>(a);
     if (launches) *launches += 2;
-    return cudaGetLastError();
+    return launch_finalize(a, s);
 }
 
 cudaError_t launch_fill(float *p, long long n, float v, cudaStream_t s)

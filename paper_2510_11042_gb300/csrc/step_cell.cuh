@@ -263,14 +263,11 @@ struct FloatCell {
 // dft_flush_x: an FP64 read-modify-write in the step holds a warp, and in the
 // two-step kernel a whole tile, for a DRAM round trip and an FP64 pass (64^3
 // FP32 single steps in the window: 23.4 us a step with only the x faces staged,
-// now 15.1).  kStaged tests for a face first and stores straight-line;
-// kStagedByFace loops over the faces, which leaves the issue-bound 16-bit
-// two-step kernel faster (384^3 FP16 outside / in the window 0.896 / 0.957 ms
-// against 0.917 / 0.962; FP32 1.549 / 1.625 against 1.555 / 1.586 the other way).
+// 15.1 with all of them).  kStaged tests for a face first and stores straight-line.
 // kDirect adds to the accumulators in place: the batched kernel, and grids
 // whose faces are too large to stage -- in a kernel of its own, for with both
 // forms in one the 16-bit single steps spilled (300^3 BF16 in place 778 -> 858 us).
-constexpr int kStaged = 0, kStagedByFace = 1, kDirect = 2;
+constexpr int kStaged = 0, kDirect = 1;
 
 // The fields of a face cell into its slot of the staged step (element j of
 // xs_n; the host keeps 8 staged steps below 2^31 elements).
@@ -349,9 +346,6 @@ __device__ __forceinline__ void update_cell(Cell &f, int x, int y, int z, float 
         on_face = on_face && (x == a.ft_lo[0] || x == a.ft_hi[0] || y == a.ft_lo[1] || y == a.ft_hi[1] ||
                               z == a.ft_lo[2] || z == a.ft_hi[2]);
     on_face = on_face && in_box(x, y, z, a.nt_lo, a.nt_hi);
-    if constexpr (MODE == 2 && FORM == kStagedByFace)
-        on_face = on_face && (x == a.nt_lo[0] || x == a.nt_hi[0] || y == a.nt_lo[1] || y == a.nt_hi[1] ||
-                              z == a.nt_lo[2] || z == a.nt_hi[2]);
     if (on_face) {
         float vals[PL::NC];
 #pragma unroll
@@ -378,12 +372,6 @@ __device__ __forceinline__ void update_cell(Cell &f, int x, int y, int z, float 
                     const int ua = ax == 2 ? 1 : 2, va = ax == 0 ? 1 : 0;
                     const int iu = g[ua] - a.nt_lo[ua], iv = g[va] - a.nt_lo[va];
                     const int nu = a.face_nu[face], nv = a.face_nv[face];
-                    if constexpr (MODE == 2 && FORM == kStagedByFace) {
-                        const long long j = a.xs_start[face] + (long long)iu * nv + iv;
-#pragma unroll
-                        for (int k = 0; k < PL::NC; ++k) a.xstage[(long long)k * a.xs_n + j] = vals[k];
-                        continue;
-                    }
                     double *base = a.dft + a.face_off[face] + (long long)iu * nv + iv;
                     const long long plane = (long long)nu * nv;
 #pragma unroll
