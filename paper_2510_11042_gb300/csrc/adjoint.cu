@@ -44,7 +44,7 @@ constexpr int kAdjBX = 128;
 // each group starting at plane slot i * NC + s0, so a group is one float2 load.
 __device__ __forceinline__ float2 ld_pair(const float *p, int k)
 {
-    return __ldg(reinterpret_cast<const float2 *>(p) + k);
+    return reinterpret_cast<const float2 *>(p)[k];
 }
 
 template <int MODE>
@@ -97,8 +97,8 @@ __global__ void __launch_bounds__(kAdjBX, MODE == 2 ? 7 : 1) adjoint_step_kernel
             m[slot_plane(MODE, i, s0 + 1)] = keep * v.y;
         }
         if (NC & 1) {
-            float v = has_nb[i] ? __ldg(g[NC - 1] + nb[i]) : 0.f;
-            if (self[i]) v += __ldg(g[NC - 1] + c);
+            float v = has_nb[i] ? g[NC - 1][nb[i]] : 0.f;
+            if (self[i]) v += g[NC - 1][c];
             m[slot_plane(MODE, i, NC - 1)] = keep * v;
         }
     }
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(kAdjBX, MODE == 2 ? 7 : 1) adjoint_step_kernel
     // this step's term in FP32 (its factors are FP32), the sum over steps in FP64
     float gs = 0.f;
 #pragma unroll
-    for (int k = 0; k < PL::NE; ++k) gs = fmaf(A[M::ec(k)], __ldg(a.rec + (long long)k * a.P + c), gs);
+    for (int k = 0; k < PL::NE; ++k) gs = fmaf(A[M::ec(k)], a.rec[(long long)k * a.P + c], gs);
     a.grad[c] += (double)gs;
 
     const float beta = __ldg(a.inv_eps + c);

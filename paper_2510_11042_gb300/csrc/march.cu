@@ -78,7 +78,7 @@ __device__ __forceinline__ void update2(const MarchArgs &a, P2 *f, int lev, cons
                 const int sl = a.inc_axis == 0 ? x : r;
 #pragma unroll
                 for (int s = 0; s < NE; ++s) {
-                    const float inc = in ? __ldg(a.lm[lev] + (size_t)s * a.n_line + sl) : 0.f;
+                    const float inc = in ? a.lm[lev][(size_t)s * a.n_line + sl] : 0.f;
                     a.rec[lev][(long long)s * a.P + (long long)r * a.nxp + x] = (c ? un(m[s]).y : un(m[s]).x) * a.scale + inc;
                 }
             }
@@ -148,8 +148,8 @@ __device__ __forceinline__ void update2(const MarchArgs &a, P2 *f, int lev, cons
             if (!e && !MU) continue;
             const float *lm = a.lm[lev] + (size_t)s * a.n_line;
             float v0 = 0.f, v1 = 0.f;
-            if (s0) v0 = __ldg(lm + l0) * (((e ? ie.x : im.x) - 1.0f) * a.inv_scale);
-            if (s1) v1 = __ldg(lm + l1) * (((e ? ie.y : im.y) - 1.0f) * a.inv_scale);
+            if (s0) v0 = lm[l0] * (((e ? ie.x : im.x) - 1.0f) * a.inv_scale);
+            if (s1) v1 = lm[l1] * (((e ? ie.y : im.y) - 1.0f) * a.inv_scale);
             d[s] = pk(v0, v1);
             d3[s] = third2(d[s]);
         }

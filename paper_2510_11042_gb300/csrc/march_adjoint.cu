@@ -217,10 +217,10 @@ __global__ void __launch_bounds__(32 * kRows, 1) march_adjoint_kernel(const __gr
                         own = r == 0 ? d[3] : d[4];
                     } else {
                         const long long c = (long long)r * a.nxp + xc;
-                        const float4 v = __ldg(reinterpret_cast<const float4 *>(a.lin[2 * i] + 2 * c));
+                        const float4 v = *reinterpret_cast<const float4 *>(a.lin[2 * i] + 2 * c);
                         own.c[0] = pk(v.x, v.z);
                         own.c[1] = pk(v.y, v.w);
-                        own.c[2] = __ldg(reinterpret_cast<const P2 *>(a.lin[2 * i + 1] + c));
+                        own.c[2] = *reinterpret_cast<const P2 *>(a.lin[2 * i + 1] + c);
                     }
                 }
                 if (l > 0) {

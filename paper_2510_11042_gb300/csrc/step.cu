@@ -63,7 +63,8 @@ namespace {
 // in-group offset from a constant-bank base; the +-x pulls are plain loads
 // shifted by one element (coalesced; the extra sector per warp hits in L1/L2).
 // The cells x = bx * blockDim.x + threadIdx.x of row (y, z) for one step.
-template <int MODE, class S, int BX, bool REC = false, bool MU = false, bool ANA = false, int FORM = kStaged>
+template <int MODE, class S, int BX, bool REC = false, bool MU = false, bool ANA = false, int FORM = kStaged,
+          bool NCL = false>
 __device__ __forceinline__ void row_cells(const StepArgs &a, int bx, int y, int z)
 {
     using PL = Planes<MODE>;
@@ -83,10 +84,10 @@ __device__ __forceinline__ void row_cells(const StepArgs &a, int bx, int y, int 
     src[6] = c + (z < a.nz - 1 ? pz : 0);
 
     float f[Q];
-    load_cell<MODE, S>(a, src, f);
+    load_cell<MODE, S, NCL>(a, src, f);
     FloatCell cell{f};
-    update_cell<MODE, REC, MU, ANA, FORM>(cell, x, y, z, __ldg(a.inv_eps + c), a,
-                                    MU ? __ldg(a.inv_mu + c) : 1.0f);
+    update_cell<MODE, REC, MU, ANA, FORM, true, NCL>(cell, x, y, z, __ldg(a.inv_eps + c), a,
+                                               MU ? __ldg(a.inv_mu + c) : 1.0f);
     store_cell<MODE, S>(a, c, f);
 }
 
@@ -100,6 +101,9 @@ __device__ __forceinline__ void row_cells(const StepArgs &a, int bx, int y, int 
 // 2.83 ms at 384^3, against 3.98 ms spilling at 7).  These were chosen by timing
 // the 384^3 sphere and 256^2 to 4096^2 EZ grids on GB300.
 template <class S> __host__ __device__ constexpr int rows_of() { return sizeof(S) == 4 ? 2 : 4; }
+
+// Whether the kernel loads through the read-only path, and so is never chained.
+template <class S, bool ONE> __host__ __device__ constexpr bool read_only_path() { return sizeof(S) == 2 && !ONE; }
 
 template <int MODE, class S, int BX, bool REC = false, bool MU = false, bool ANA = false, bool ONE = false,
           int FORM = kStaged>
@@ -117,7 +121,8 @@ __global__ void __launch_bounds__(BX, (ANA && MODE == 2) ? 5 : 7) step_kernel_ce
     const int bx = tile % a.nblk_x;
     const int r0 = (tile / a.nblk_x) * R;
     const int r1 = min(r0 + R, a.ny * a.nz);
-    for (int r = r0; r < r1; ++r) row_cells<MODE, S, BX, REC, MU, ANA, FORM>(a, bx, r % a.ny, r / a.ny);
+    for (int r = r0; r < r1; ++r)
+        row_cells<MODE, S, BX, REC, MU, ANA, FORM, read_only_path<S, ONE>()>(a, bx, r % a.ny, r / a.ny);
 }
 
 constexpr int kBX = 128;  // threads per block at most; cells per row tile of the batched kernel
@@ -333,7 +338,7 @@ cudaError_t launch_cell(StepArgs a, cudaStream_t s)
     }
     if (a.rows_per_block == 1)
         return launch_chained(a.chain != 0, step_kernel_cell<MODE, S, kBX, REC, MU, ANA, true>, a.nblk_main, tx, 0, s, a);
-    return launch_chained(a.chain != 0, step_kernel_cell<MODE, S, kBX, REC, MU, ANA, false>, a.nblk_main, tx, 0, s, a);
+    return launch_chained(a.chain != 0 && !read_only_path<S, false>(), step_kernel_cell<MODE, S, kBX, REC, MU, ANA, false>, a.nblk_main, tx, 0, s, a);
 }
 
 template <int MODE, class S>

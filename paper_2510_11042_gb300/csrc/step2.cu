@@ -411,7 +411,7 @@ __device__ __forceinline__ void t2_level2(const StepArgs &s2, const unsigned cha
     from_dir<S>(d5, f, 5);
     from_dir<S>(d6, f, 6);
     FloatCell cell{f};
-    update_cell<2, false, (V > 0), false, kStaged>(cell, x, y, z, ie, s2, im, true);
+    update_cell<2, false, (V > 0), false, kStaged, true, true>(cell, x, y, z, ie, s2, im, true);
     store_cell_evict_first<S>(s2, (z * ny + y) * s2.nxp + x, f);
 }
 
@@ -489,7 +489,7 @@ __device__ __forceinline__ void step2_body(const Step2Args &P)
             float im = 1.f;
             if constexpr (L::HAS_MU) im = reinterpret_cast<const float *>(buf + L::MU_OFF)[ei];
             FloatCell cell{f};
-            update_cell<2, false, (V > 0), false, kStaged>(cell, x, y, p, ie, s1, im, tile && p >= z0 && p < z1);
+            update_cell<2, false, (V > 0), false, kStaged, true, true>(cell, x, y, p, ie, s1, im, tile && p >= z0 && p < z1);
             if (tile) {
 #pragma unroll
                 for (int d = 1; d <= 4; ++d) slot_put<S>(slot, false, d, t, to_dir<S>(f, d));

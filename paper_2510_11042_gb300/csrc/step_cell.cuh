@@ -64,7 +64,7 @@ __device__ __forceinline__ void collide(float *f, const float D[3], const float 
 // (pull along the line with the clamped ends, eps_r = 1 moments and collision,
 // absorbing layer at both ends, hard source overwrite at src_index).
 template <int MODE>
-__device__ __noinline__ void line_node(const float *__restrict__ line_in, float *__restrict__ line_out,
+__device__ __noinline__ void line_node(const float *line_in, float *line_out,
                                        int n, int s, int w, float sigma_max, float inv_w,
                                        int src_index, float sE0, float sE1, float sE2, float sH0,
                                        float sH1, float sH2, int axis)
@@ -259,6 +259,20 @@ struct FloatCell {
     __device__ __forceinline__ void set(int q, float v) { f[q] = v; }
 };
 
+// A value that an earlier kernel, or an earlier step of the same kernel, wrote.
+// NCL reads it through the read-only path, which is for data that no one writes
+// while the kernel lives.  A chained kernel (launch_chained) lives before the one
+// before it has finished, and the batched kernel through many steps: they read
+// plainly.  Plain loads don't move over the stores of a block's row before:
+// 16-bit single steps, which take four rows a block, keep the read-only path
+// and are not chained (300^3 FP16 719 -> 694 us, 96^3 24.4), and so do two-step
+// passes (384^3 FP16 859 -> 849 us).
+template <bool NCL, class T> __device__ __forceinline__ T load_value(const T *p)
+{
+    if constexpr (NCL) return __ldg(p);
+    else return *p;
+}
+
 // The running DFT of cells on the NTFF box, in 3D.  Kernels stage the fields for
 // dft_flush_x: an FP64 read-modify-write in the step holds a warp, and in the
 // two-step kernel a whole tile, for a DRAM round trip and an FP64 pass (64^3
@@ -284,7 +298,7 @@ template <int NC> __device__ __forceinline__ void stage_fields(const StepArgs &a
 // multiplied back by the scale (dft_scale_cells), the incident source is
 // divided by it.
 template <int MODE, bool REC = false, bool MU = false, bool ANA = false, int FORM = kStaged, bool EARLY = true,
-          class Cell>
+          bool NCL = false, class Cell>
 __device__ __forceinline__ void update_cell(Cell &f, int x, int y, int z, float inv_eps,
                                             const StepArgs &a, float inv_mu = 1.0f, bool surface = true)
 {
@@ -323,7 +337,7 @@ __device__ __forceinline__ void update_cell(Cell &f, int x, int y, int z, float 
             const int sl = a.inc_axis == 0 ? x : (a.inc_axis == 1 ? y : z);
 #pragma unroll
             for (int q = 0; q < 7 * PL::NE; ++q)
-                Dinc[PL::comp(q)] += __ldg(a.line_n1 + (size_t)q * a.n_line + sl);
+                Dinc[PL::comp(q)] += load_value<NCL>(a.line_n1 + (size_t)q * a.n_line + sl);
         }
         const long long c = ((long long)z * a.ny + y) * a.nxp + x;
 #pragma unroll
@@ -448,7 +462,7 @@ __device__ __forceinline__ void update_cell(Cell &f, int x, int y, int z, float 
         const int sl = a.inc_axis == 0 ? x : (a.inc_axis == 1 ? y : z);
 #pragma unroll
         for (int q = 0; q < 7 * PL::NE; ++q)
-            dE[PL::comp(q)] += __ldg(a.line_n1 + (size_t)q * a.n_line + sl);
+            dE[PL::comp(q)] += load_value<NCL>(a.line_n1 + (size_t)q * a.n_line + sl);
         const float g = (inv_eps - 1.0f) * a.inv_scale;  // to storage units
 #pragma unroll
         for (int c3 = 0; c3 < 3; ++c3) {
@@ -458,7 +472,7 @@ __device__ __forceinline__ void update_cell(Cell &f, int x, int y, int z, float 
         if (MU) {
 #pragma unroll
             for (int q = 7 * PL::NE; q < Q; ++q)
-                dH[PL::comp(q)] += __ldg(a.line_n1 + (size_t)q * a.n_line + sl);
+                dH[PL::comp(q)] += load_value<NCL>(a.line_n1 + (size_t)q * a.n_line + sl);
             const float gh = (inv_mu - 1.0f) * a.inv_scale;
 #pragma unroll
             for (int c3 = 0; c3 < 3; ++c3) {
@@ -492,15 +506,16 @@ __device__ __forceinline__ void update_cell(Cell &f, int x, int y, int z, float 
 // Vector access to one group of a cell's populations (the storage layout is
 // described with pop_index): W = 1, 2 or 4 consecutive slots in one load or
 // store, converted to or from FP32; 16-bit pairs use the paired conversions.
-template <class S> struct Io;
-template <> struct Io<float> {
+// NCL: through the read-only path (load_value).
+template <class S, bool NCL = false> struct Io;
+template <bool NCL> struct Io<float, NCL> {
     static __device__ __forceinline__ void ld1(const void *p, int k, float &a)
     {
-        a = __ldg(static_cast<const float *>(p) + k);
+        a = load_value<NCL>(static_cast<const float *>(p) + k);
     }
     static __device__ __forceinline__ void ld2(const void *p, int k, float &a, float &b)
     {
-        const float2 v = __ldg(static_cast<const float2 *>(p) + k);
+        const float2 v = load_value<NCL>(static_cast<const float2 *>(p) + k);
         a = v.x;
         b = v.y;
     }
@@ -510,7 +525,7 @@ template <> struct Io<float> {
         static_cast<float2 *>(p)[k] = make_float2(a, b);
     }
 };
-template <class H, class H2> struct Io16 {
+template <class H, class H2, bool NCL> struct Io16 {
     static __device__ __forceinline__ float2 unpack(unsigned u)
     {
         H2 h;
@@ -529,19 +544,19 @@ template <class H, class H2> struct Io16 {
     }
     static __device__ __forceinline__ void ld1(const void *p, int k, float &a)
     {
-        const H v = __ldg(static_cast<const H *>(p) + k);
+        const H v = load_value<NCL>(static_cast<const H *>(p) + k);
         if constexpr (std::is_same<H, __half>::value) a = __half2float(v);
         else a = __bfloat162float(v);
     }
     static __device__ __forceinline__ void ld2(const void *p, int k, float &a, float &b)
     {
-        const float2 v = unpack(__ldg(static_cast<const unsigned *>(p) + k));
+        const float2 v = unpack(load_value<NCL>(static_cast<const unsigned *>(p) + k));
         a = v.x;
         b = v.y;
     }
     static __device__ __forceinline__ void ld4(const void *p, int k, float &a, float &b, float &c, float &d)
     {
-        const uint2 u = __ldg(static_cast<const uint2 *>(p) + k);
+        const uint2 u = load_value<NCL>(static_cast<const uint2 *>(p) + k);
         const float2 v0 = unpack(u.x), v1 = unpack(u.y);
         a = v0.x;
         b = v0.y;
@@ -562,8 +577,8 @@ template <class H, class H2> struct Io16 {
         static_cast<uint2 *>(p)[k] = make_uint2(pack(a, b), pack(c, d));
     }
 };
-template <> struct Io<__half> : Io16<__half, __half2> {};
-template <> struct Io<__nv_bfloat16> : Io16<__nv_bfloat16, __nv_bfloat162> {};
+template <bool NCL> struct Io<__half, NCL> : Io16<__half, __half2, NCL> {};
+template <bool NCL> struct Io<__nv_bfloat16, NCL> : Io16<__nv_bfloat16, __nv_bfloat162, NCL> {};
 
 // Threads of a single step's block, one per cell of a row tile: 128, 96 or 64,
 // the widest of those that leave the fewest lanes beyond the row's end (idle
@@ -579,7 +594,7 @@ inline int row_threads(int nx)
 
 // All populations of one cell: direction i's groups read at cell index src[i]
 // (load) or written at c (store); f is indexed by population plane.
-template <int MODE, class S>
+template <int MODE, class S, bool NCL>
 __device__ __forceinline__ void load_cell(const StepArgs &a, const int src[7], float *f)
 {
     constexpr int NC = Planes<MODE>::NC;
@@ -588,15 +603,15 @@ __device__ __forceinline__ void load_cell(const StepArgs &a, const int src[7], f
     for (int i = 0; i < 7; ++i) {
         const void *const *b = a.fin_q + i * NC;
         if constexpr (NC == 3) {
-            Io<S>::ld2(b[0], src[i], SQ(0), SQ(1));
-            Io<S>::ld1(b[2], src[i], SQ(2));
+            Io<S, NCL>::ld2(b[0], src[i], SQ(0), SQ(1));
+            Io<S, NCL>::ld1(b[2], src[i], SQ(2));
         } else if constexpr (sizeof(S) == 4) {
-            Io<S>::ld2(b[0], src[i], SQ(0), SQ(1));
-            Io<S>::ld2(b[2], src[i], SQ(2), SQ(3));
-            Io<S>::ld2(b[4], src[i], SQ(4), SQ(5));
+            Io<S, NCL>::ld2(b[0], src[i], SQ(0), SQ(1));
+            Io<S, NCL>::ld2(b[2], src[i], SQ(2), SQ(3));
+            Io<S, NCL>::ld2(b[4], src[i], SQ(4), SQ(5));
         } else {
-            Io<S>::ld4(b[0], src[i], SQ(0), SQ(1), SQ(2), SQ(3));
-            Io<S>::ld2(b[4], src[i], SQ(4), SQ(5));
+            Io<S, NCL>::ld4(b[0], src[i], SQ(0), SQ(1), SQ(2), SQ(3));
+            Io<S, NCL>::ld2(b[4], src[i], SQ(4), SQ(5));
         }
     }
 }
