@@ -62,9 +62,13 @@ namespace {
 // a.fin_q[i * NC + s0] (kernel parameters), so every access is a 32-bit
 // in-group offset from a constant-bank base; the +-x pulls are plain loads
 // shifted by one element (coalesced; the extra sector per warp hits in L1/L2).
-// The cells x = bx * blockDim.x + threadIdx.x of row (y, z) for one step.
+// The cells x = bx * blockDim.x + threadIdx.x of row (y, z) for one step.  WAIT
+// (closed-form source, 2D): what does not need the populations, the eight wave
+// evaluations above all, comes before the wait for the kernel before this one
+// (chain_wait): 200^2 EZ 4.9 -> 3.2 us a step.  In 3D the terms' registers beside
+// 42 populations would spill.
 template <int MODE, class S, int BX, bool REC = false, bool MU = false, bool ANA = false, int FORM = kStaged,
-          bool NCL = false>
+          bool NCL = false, bool WAIT = false>
 __device__ __forceinline__ void row_cells(const StepArgs &a, int bx, int y, int z)
 {
     using PL = Planes<MODE>;
@@ -83,11 +87,16 @@ __device__ __forceinline__ void row_cells(const StepArgs &a, int bx, int y, int 
     src[5] = c - (z > 0 ? pz : 0);
     src[6] = c + (z < a.nz - 1 ? pz : 0);
 
+    const float ie = __ldg(a.inv_eps + c), im = MU ? __ldg(a.inv_mu + c) : 1.0f;
+    AnaTerms<MODE> terms;
+    if constexpr (WAIT) {
+        if (in_box(x, y, z, a.tf_lo, a.tf_hi)) analytic_prepare<MODE>(a, x, y, z, ie, im, cell_keep(a, x, y, z), terms);
+        chain_wait();
+    }
     float f[Q];
     load_cell<MODE, S, NCL>(a, src, f);
     FloatCell cell{f};
-    update_cell<MODE, REC, MU, ANA, FORM, true, NCL>(cell, x, y, z, __ldg(a.inv_eps + c), a,
-                                               MU ? __ldg(a.inv_mu + c) : 1.0f);
+    update_cell<MODE, REC, MU, ANA, FORM, true, NCL>(cell, x, y, z, ie, a, im, true, WAIT ? &terms : nullptr);
     store_cell<MODE, S>(a, c, f);
 }
 
@@ -110,9 +119,10 @@ template <int MODE, class S, int BX, bool REC = false, bool MU = false, bool ANA
 __global__ void __launch_bounds__(BX, (ANA && MODE == 2) ? 5 : 7) step_kernel_cell(const StepArgs a)
 {
     constexpr int R = ONE ? 1 : rows_of<S>();
+    constexpr bool WAIT = ANA && ONE && MODE != 2;
     const int b = blockIdx.x;
     chain_release();
-    chain_wait();
+    if (!WAIT) chain_wait();
     if (a.line_on) {
         const int s = b * blockDim.x + threadIdx.x;
         if (s < a.n_line) line_work<MODE>(a, s);
@@ -122,7 +132,7 @@ __global__ void __launch_bounds__(BX, (ANA && MODE == 2) ? 5 : 7) step_kernel_ce
     const int r0 = (tile / a.nblk_x) * R;
     const int r1 = min(r0 + R, a.ny * a.nz);
     for (int r = r0; r < r1; ++r)
-        row_cells<MODE, S, BX, REC, MU, ANA, FORM, read_only_path<S, ONE>()>(a, bx, r % a.ny, r / a.ny);
+        row_cells<MODE, S, BX, REC, MU, ANA, FORM, read_only_path<S, ONE>(), WAIT>(a, bx, r % a.ny, r / a.ny);
 }
 
 constexpr int kBX = 128;  // threads per block at most; cells per row tile of the batched kernel

@@ -252,6 +252,15 @@ __device__ __forceinline__ float analytic_term(const StepArgs &a, const AnaTerms
     return (t.h3[c] + cross_c(i, t.e3, c)) - t.b[i] * ((kxp[c] + cross_c(i, pol, c)) * sixth);
 }
 
+// The absorbing layer's factor of a cell.
+__device__ __forceinline__ float cell_keep(const StepArgs &a, int x, int y, int z)
+{
+    int d = min(x, a.nx - 1 - x);
+    d = min(d, min(y, a.ny - 1 - y));
+    if (a.nz > 1) d = min(d, min(z, a.nz - 1 - z));
+    return layer_keep(d, a.w, a.sigma_max, a.inv_w);
+}
+
 // Accessor of one cell's pulled populations held in registers.
 struct FloatCell {
     float *f;
@@ -296,11 +305,13 @@ template <int NC> __device__ __forceinline__ void stage_fields(const StepArgs &a
 //   f* = (2 f_eq - f + source) * keep.
 // Values are in storage units (population / scale); fields go to the DFT
 // multiplied back by the scale (dft_scale_cells), the incident source is
-// divided by it.
+// divided by it.  terms: the closed-form source's terms of the cell, where the
+// caller has them.
 template <int MODE, bool REC = false, bool MU = false, bool ANA = false, int FORM = kStaged, bool EARLY = true,
           bool NCL = false, class Cell>
 __device__ __forceinline__ void update_cell(Cell &f, int x, int y, int z, float inv_eps,
-                                            const StepArgs &a, float inv_mu = 1.0f, bool surface = true)
+                                            const StepArgs &a, float inv_mu = 1.0f, bool surface = true,
+                                            const AnaTerms<MODE> *terms = nullptr)
 {
     using PL = Planes<MODE>;
     using M = Mode<MODE>;
@@ -404,10 +415,7 @@ __device__ __forceinline__ void update_cell(Cell &f, int x, int y, int z, float 
 #pragma unroll
     for (int k = 0; k < PL::NH; ++k) H3[M::hc(k)] = third(H[M::hc(k)]);
 
-    int d = min(x, a.nx - 1 - x);
-    d = min(d, min(y, a.ny - 1 - y));
-    if (a.nz > 1) d = min(d, min(z, a.nz - 1 - z));
-    const float keep = layer_keep(d, a.w, a.sigma_max, a.inv_w);
+    const float keep = cell_keep(a, x, y, z);
 
     // incident-field source of dielectric cells inside the total-field box
     // (the box lies outside the absorbing layer, so keep == 1 there)
@@ -496,7 +504,8 @@ __device__ __forceinline__ void update_cell(Cell &f, int x, int y, int z, float 
     if constexpr (ANA) {
         if (ana) {
             AnaTerms<MODE> at;
-            analytic_prepare<MODE>(a, x, y, z, inv_eps, inv_mu, keep, at);
+            if (terms) at = *terms;
+            else analytic_prepare<MODE>(a, x, y, z, inv_eps, inv_mu, keep, at);
 #pragma unroll
             for (int q = 0; q < Q; ++q) f.set(q, f.get(q) + analytic_term<MODE>(a, at, q));
         }
