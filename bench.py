@@ -60,11 +60,11 @@ def b_cell(mode: str, storage: str) -> int:
 
 
 def kernel_source_hash() -> str:
-    """Hash of the step kernels' source: step.cu, step2.cu, step_cell.cuh and
-    the StepArgs definition."""
+    """Hash of the step kernels' source: step.cu, step2.cu, march.cu, march.cuh,
+    step_cell.cuh and the StepArgs definition."""
     csrc = os.path.join(ROOT, "paper_2510_11042_gb300", "csrc")
     h = hashlib.sha256()
-    for name in ("step.cu", "step2.cu", "step_cell.cuh"):
+    for name in ("step.cu", "step2.cu", "march.cu", "march.cuh", "step_cell.cuh"):
         with open(os.path.join(csrc, name), "rb") as fh:
             h.update(fh.read())
     hdr = open(os.path.join(csrc, "lbem_internal.cuh")).read()
@@ -483,8 +483,7 @@ def run_probe_2d(dev, n=4096, updates=60):
     """Step throughput of the 2D EZ path on a grid well above L2 (4096^2 x 21
     populations, 2.8 GB in FP32): a cylinder of the cylinder workload's
     proportions, CUDA events around `updates` lattice updates, with the pass
-    lbem_step takes by default (two updates per pass where the library
-    reports it) and with single steps.  hbm_frac is the byte model
+    lbem_step takes by default (four updates per pass) and with single steps.  hbm_frac is the byte model
     (B_cell per update) over the time per update."""
     import torch
     from paper_2510_11042_gb300 import lbem
@@ -515,10 +514,10 @@ def run_probe_2d(dev, n=4096, updates=60):
             torch.cuda.empty_cache()
         out[st] = dict(rec[2], single_step=rec[1], speedup_vs_single_step=round(rec[1]["kernel_ms"] /
                                                                                 rec[2]["kernel_ms"], 3))
-        # the two-step kernel's own DRAM traffic (ncu, committed summary), over the time of its launch
+        # the four-step kernel's own DRAM traffic (ncu, committed summary), over the time of its launch
         traffic = traffic_from_profile(f"cylinder_{n}_ez", st) if rec[2]["steps_per_pass"] == 2 else None
         if traffic:
-            gbs_t = traffic / (2 * rec[2]["kernel_ms"] / 1e3) / 1e9
+            gbs_t = traffic / (4 * rec[2]["kernel_ms"] / 1e3) / 1e9
             out[st]["dram_traffic_per_launch"] = traffic
             out[st]["dram_traffic_gbs"] = round(gbs_t, 1)
             out[st]["dram_traffic_frac"] = round(gbs_t / hbm, 4)
@@ -529,7 +528,7 @@ def run_probe_2d(dev, n=4096, updates=60):
 def run_cylinder_1024(dev, updates=120):
     """Step throughput on the cylinder workload itself (1024^2, a = 31.83,
     eps_r = 2.25, W = 20, TM and TE) over one DFT window of 120 updates, with
-    the pass lbem_step takes (single steps: two 1024^2 buffers stay in L2).
+    the pass lbem_step takes (four steps).
     The byte model's fraction is labelled L2-assisted where the working set is
     under three times the L2 size."""
     import torch

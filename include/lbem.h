@@ -223,24 +223,25 @@ int32_t lbem_set_permeability(lbem_handle h, const float *mu_r, int32_t mu_on_de
 int32_t lbem_far_field(lbem_handle h, const double *theta_host, const double *phi_host,
                        int32_t n, double *s2_host, double *amp_host);
 
-/* Temporal blocking (Eq. 1 applied twice per pass over memory):
+/* Temporal blocking (Eq. 1 applied several times per pass over memory):
  * steps_per_pass = 2 (the default) lets lbem_step advance grids of any mode
- * and storage, with or without a mu_r map, two steps per pass over the
- * populations: a fused kernel keeps the intermediate state of each tile (3D:
- * 32 x 8 cells in FP32, 32 x 16 in FP16/BF16, marching through a chunk of z
- * planes; 2D: 128-cell strips marching along y) plus its edge halos in shared
- * memory, bitwise the same result as two single steps (16-bit storage rounds
- * the intermediate state as a single step stores it).  It is taken where its
- * blocks fill the GPU (one wave of resident blocks in 3D, two in 2D) and, in
- * 2D, where the population buffers of the grids stepping together outgrow
- * the L2 cache (smaller grids are served from it); other grids, the
- * closed-form source (bound by its wave evaluations, not by memory), a last
- * odd step and handles with in-place streaming take single steps.
+ * and storage, with or without a mu_r map, several steps per pass over the
+ * populations, bitwise the same result as single steps (16-bit storage rounds
+ * the states between as a single step stores them).  In 3D a pass takes two
+ * steps: a fused kernel keeps the intermediate state of each tile (32 x 8
+ * cells in FP32, 32 x 16 in FP16/BF16, marching through a chunk of z planes)
+ * plus its edge halos in shared memory; it is taken where its blocks fill the
+ * GPU (one wave of resident blocks).  In 2D a pass takes four steps, on every
+ * grid of at least 2 x 2 cells: strips of 56 cells march along y with a row's
+ * levels in registers.  Other grids, the closed-form source (bound by its
+ * wave evaluations, not by memory), the steps a pass leaves over and handles
+ * with in-place streaming take single steps.
  * 1 always takes single steps.  Anything else: LBEM_ERR_ARG. */
 int32_t lbem_set_step_fusion(lbem_handle h, int32_t steps_per_pass);
 
-/* The steps per pass lbem_step takes on this handle as it is now configured:
- * 2 where two-step passes apply (see lbem_set_step_fusion), else 1.
+/* Whether lbem_step takes several steps per pass on this handle as it is now
+ * configured, as the value lbem_set_step_fusion takes: 2 where it does (two
+ * steps in 3D, four in 2D), else 1.
  * NULL argument: LBEM_ERR_ARG. */
 int32_t lbem_get_step_fusion(lbem_handle h, int32_t *steps_per_pass);
 
