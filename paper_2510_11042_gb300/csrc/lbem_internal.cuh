@@ -29,8 +29,8 @@ long long l2_bytes();
 // global memory that others write, and reads it by plain loads (the read-only path
 // is for data that does not change while the kernel lives); chain_release() lets
 // the next one be scheduled.  us a step, plain -> chained: 200^2 with the
-// closed-form source 6.2 -> 4.9 (-> 3.2 with the source formed before the wait), 520^2 HZ 4.7 -> 4.3, 64^3 FP32 12.5 -> 11.2, 512^2
-// adjoint 11.6 -> 10.5.
+// closed-form source 6.2 -> 4.9 (3.2 with the source formed before the wait),
+// 520^2 HZ 4.7 -> 4.3, 64^3 FP32 12.5 -> 11.2, 512^2 adjoint 11.6 -> 10.5.
 template <class... P, class... A>
 cudaError_t launch_chained(bool chain, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                            A &&...args)
