@@ -59,17 +59,18 @@ def b_cell(mode: str, storage: str) -> int:
     return 2 * q * s + 4
 
 
-def kernel_source_hash() -> str:
-    """Hash of the step kernels' source: step.cu, step2.cu, march.cu, march.cuh,
-    step_cell.cuh and the StepArgs definition."""
+def kernel_source_hash(two_d: bool = False) -> str:
+    """Hash of the step kernels' source: in 3D step.cu, step2.cu, step_cell.cuh
+    and the StepArgs definition, in 2D march.cu and march.cuh."""
     csrc = os.path.join(ROOT, "paper_2510_11042_gb300", "csrc")
     h = hashlib.sha256()
-    for name in ("step.cu", "step2.cu", "march.cu", "march.cuh", "step_cell.cuh"):
+    for name in ("march.cu", "march.cuh") if two_d else ("step.cu", "step2.cu", "step_cell.cuh"):
         with open(os.path.join(csrc, name), "rb") as fh:
             h.update(fh.read())
-    hdr = open(os.path.join(csrc, "lbem_internal.cuh")).read()
-    i = hdr.index("struct StepArgs {")
-    h.update(hdr[i:hdr.index("};", i)].encode())
+    if not two_d:
+        hdr = open(os.path.join(csrc, "lbem_internal.cuh")).read()
+        i = hdr.index("struct StepArgs {")
+        h.update(hdr[i:hdr.index("};", i)].encode())
     return h.hexdigest()[:16]
 
 
@@ -81,7 +82,7 @@ def traffic_from_profile(workload: str, storage: str):
         with open(path) as fh:
             d = json.load(fh)
         e = d[workload][storage]
-        if e.get("kernel_hash") != kernel_source_hash():
+        if e.get("kernel_hash") != kernel_source_hash(workload.startswith("cylinder")):
             return None
         return float(e["bytes_per_launch"])
     except Exception:
