@@ -1147,7 +1147,12 @@ static int step_loop(lbem_ctx *h, int64_t n)
     if (pairs) fill_common_args(h, a2);
     MarchArgs m;
     if (march) march_common(h, m);
+    // The call's first step is launched plainly, behind whatever wrote the maps,
+    // the state and the line before; the others chain to the step before them.
+    const int chain = a.chain;
     for (int64_t k = 0; k < n;) {
+        a.chain = k > 0 ? chain : 0;
+        m.chain = k > 0;
         if (march && n - k >= kMarchSteps) {
             if (h->ms_cnt + kMarchSteps > h->ms_cap) {
                 const int rc = flush_march(h);
@@ -2241,6 +2246,7 @@ int32_t lbem_adjoint(lbem_handle h, const double *theta, const double *phi, cons
     StepArgs a;
     fill_common_args(h, a);
     a.dft_on = 0;
+    const int chain = a.chain;
     AdjointArgs b;
     std::memset(&b, 0, sizeof b);
     b.inv_eps = h->inv_eps;
@@ -2312,6 +2318,10 @@ int32_t lbem_adjoint(lbem_handle h, const double *theta, const double *phi, cons
         int64_t front = -1;
         for (int64_t k = 0; k < len;) {
             const int64_t t = t0 + k;   // state time before the step
+            // the sweep's first launch is plain, as lbem_step's
+            const bool behind = k > 0 || seg < L.nseg - 1;
+            a.chain = behind ? chain : 0;
+            m.chain = behind;
             if (march && len - k >= kMarchSteps) {
                 if (front != t + kMarchSteps) {
                     const int rc = march_line_start(h, m.line, rl, t, line_from(t + 1));

@@ -28,7 +28,11 @@ long long l2_bytes();
 // are visible.  Every kernel launched so calls chain_wait() before it touches
 // global memory that others write, and reads it by plain loads (the read-only path
 // is for data that does not change while the kernel lives); chain_release() lets
-// the next one be scheduled.  us a step, plain -> chained: 200^2 with the
+// the next one be scheduled.  Exempt from the wait is what was complete before the
+// chain began: a chain's first kernel is launched plainly, in the call that builds
+// the chain, so 1/eps_r, 1/mu_r and the wave tables (step kernels), the angles and
+// the incident line's DFT (far_field_finalize), which no kernel of the chain
+// writes, may be read at any time.  us a step, plain -> chained: 200^2 with the
 // closed-form source 6.2 -> 4.9 (3.2 with the source formed before the wait),
 // 520^2 HZ 4.7 -> 4.3, 64^3 FP32 12.5 -> 11.2, 512^2 adjoint 11.6 -> 10.5.
 template <class... P, class... A>
@@ -273,7 +277,7 @@ struct StepArgs {
     double *line_dft;          // [n_line][3][2]
     // reduced-precision storage: stored = population / scale (power of two)
     float scale, inv_scale;
-    int chain;                 // launch chained to the kernel before it (launch_chained)
+    int chain;                 // launch chained to the kernel before it, a step of the same call (launch_chained)
     // Tiles from the last to the first, on every other step: a step then starts
     // on the cells the one before it wrote last, which L2 (129 MB) still holds,
     // where the same order each time finds only evicted lines.  us a single step,
@@ -409,6 +413,7 @@ struct MarchArgs {
     long long xs_n, xs_start[4];
     int nt_lo[2], nt_hi[2];
     float *rec[kMarchSteps];       // total-field D (adjoint replay)
+    int chain;                     // as StepArgs::chain
     LineMarch line;                // the line's steps for the next pass (steps = 0: none)
 };
 

@@ -438,7 +438,7 @@ cudaError_t launch_march_t(MarchArgs a, int share, cudaStream_t s)
     a.line_blocks = (a.line_warps + kRows - 1) / kRows;
     const long long blocks = a.line_blocks + chunks * a.strips;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    return launch_chained(share == 1, march_kernel<MODE, S, MU, REC>, (unsigned)blocks, 32 * kRows, march_smem<S, MU>(), s, a);
+    return launch_chained(a.chain != 0 && share == 1, march_kernel<MODE, S, MU, REC>, (unsigned)blocks, 32 * kRows, march_smem<S, MU>(), s, a);
 }
 
 template <int MODE>

@@ -1,0 +1,56 @@
+"""Calls that change what the steps read, taken between two of them: the step
+kernels of one call are chained (a kernel may start before the one before it has
+finished), and what the changing call enqueued has to be complete all the same.
+Both sides of each comparison run the same kernels on the same values, so the
+tolerance is equality."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import workloads as W
+from _parity import gpu_solver
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2510_11042_gb300 import lbem
+    lbem.lib()
+
+
+@pytest.mark.parametrize("mode,shape,analytic", [("ez", (200, 200, 1), True), ("hz", (131, 77, 1), True),
+                                                 ("ez", (200, 200, 1), False), ("3d", (48, 40, 36), False)])
+def test_maps_changed_between_steps(mode, shape, analytic):
+    """eps_r and mu_r maps set and followed at once by steps, against the same
+    calls with the stream synchronised after each."""
+    import torch
+    wave = W.axis_wave(mode, shape, 6, 10.0, gap_ntff=2, gap_tf=2)
+    if analytic:
+        wave = dataclasses.replace(wave, analytic=True, origin=(20.0, 20.0, 0.0))
+    eps = [torch.from_numpy(W.random_eps(shape, 1.0, 4.0, k)).cuda() for k in range(4)]
+    mu = torch.from_numpy(W.random_eps(shape, 1.0, 2.0, 9)).cuda()
+    p = W.Problem("maps", mode, shape, eps[0].cpu().numpy(), 6, 0.3, wave, 60, 1)
+    got = []
+    for wait in (True, False):
+        s = gpu_solver(p, steps=0, dft=False, init=W.random_state_f32(mode, shape, 6))
+        s.step(40)
+        for k in range(24):
+            s.set_permittivity(eps[k % 4])
+            if wait:
+                torch.cuda.synchronize()
+            s.step(2)
+            if k % 4 == 3:
+                s.set_permeability(mu if k % 8 == 3 else None)
+                if wait:
+                    torch.cuda.synchronize()
+                s.step(5)
+        s.sync()
+        got.append(s.populations())
+        s.close()
+    assert np.isfinite(got[0]).all() and np.abs(got[0]).max() > 0
+    assert np.array_equal(got[0], got[1])
