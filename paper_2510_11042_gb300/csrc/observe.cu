@@ -36,6 +36,7 @@ __device__ __forceinline__ double warp_sum(double v)
 // ------------------------------------------------------------ far field
 constexpr int kFFThreads = 256;
 constexpr int kFFTableMax = 4480;   // phase entries held in shared memory (70 KB)
+constexpr int kFFStaticMax = 1536;  // bytes of static shared memory of far_field_columns, at most (1152 in 3D)
 
 // How a block of far_field_columns gets its phases exp(j k r_a (p_a - c_a)):
 // evaluated at each use; as products of a coarse entry (every F-th coordinate)
@@ -237,6 +238,7 @@ __global__ void __launch_bounds__(kFFThreads) far_field_columns(const FarFieldAr
     const double sum = warp_scatter(v, lane);
     if (lane % (32 / N) == 0) red[wid][lane / (32 / N)] = sum;
     __syncthreads();
+    static_assert(sizeof rh + sizeof tw + sizeof red <= kFFStaticMax, "the shared-memory opt-in counts them");
     if (threadIdx.x < 12) {
         double s = 0.0;
 #pragma unroll
@@ -954,7 +956,8 @@ template <int MODE, int PH>
 static cudaError_t far_field_columns_go(const FarFieldArgs &a, int entries, cudaStream_t s)
 {
     const size_t smem = (size_t)entries * sizeof(double2);
-    if (smem > 47 * 1024) {
+    // static and dynamic shared memory together stay within 48 KB without the opt-in
+    if (smem + kFFStaticMax > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(far_field_columns<MODE, PH>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    kFFTableMax * (int)sizeof(double2));
