@@ -671,7 +671,7 @@ int32_t lbem_inject_plane_wave(lbem_handle h, const lbem_plane_wave *w)
     build_faces(h);
     h->dft_t0 = -1;
     h->dft_periods = 0;
-    for (int k = 0; k < 3; ++k)
+    for (int k = 0; k < kLineBufs; ++k)
         CK(h, cudaMemsetAsync(h->line[k], 0, (size_t)h->Q * h->n_line_max * 4, h->stream));
     CK(h, cudaMemsetAsync(h->line_dft, 0, (size_t)h->n_line_max * 6 * 8, h->stream));
     CK(h, cudaMemsetAsync(h->dft, 0, h->dft_doubles * 8, h->stream));

@@ -54,3 +54,33 @@ def test_maps_changed_between_steps(mode, shape, analytic):
         s.close()
     assert np.isfinite(got[0]).all() and np.abs(got[0]).max() > 0
     assert np.array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("t", [7, 8, 9, 10])
+@pytest.mark.parametrize("mode,shape", [("ez", (90, 70, 1)), ("3d", (40, 36, 34))])
+def test_a_wave_injected_again_starts_from_an_empty_line(mode, shape, t):
+    """At any time, after another wave has filled the line's buffers: as on a
+    handle that never had one, in a workspace of zeros."""
+    wave = W.axis_wave(mode, shape, 4, 10.0, gap_ntff=2, gap_tf=2)
+    first = dataclasses.replace(wave, wavelength=8.0, amplitude=3.0, ramp_periods=0.0)
+    p = W.Problem("again", mode, shape, W.random_eps(shape, 1.0, 4.0, 5), 4, 0.3, None, 60, 1)
+    init = W.random_state_f32(mode, shape, 6)
+    got = []
+    for again in (False, True):
+        s = gpu_solver(p, steps=0)
+        if again:
+            s.inject(first)
+        else:
+            s.workspace.zero_()          # and what the handle keeps there, anew
+            s.set_permittivity(p.eps)
+            s.set_permeability(None)
+        s.step(t)
+        s.inject(wave)
+        s.set_populations(init)
+        s.set_dft_window(t + 3, 1)
+        s.step(38)
+        s.sync()
+        got.append([s.populations(), s.dft(), s.incident_amplitude()])
+        s.close()
+    for a, b in zip(*got):
+        assert np.isfinite(a).all() and np.array_equal(a, b)
