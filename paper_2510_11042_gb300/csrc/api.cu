@@ -872,6 +872,12 @@ static int flush_x_stage(lbem_ctx *h, bool beside)
     return LBEM_OK;
 }
 
+// Whether the fields of time t are in the DFT window.
+static bool dft_at(const lbem_ctx *h, int64_t t)
+{
+    return h->faces.nfaces > 0 && h->dft_t0 >= 1 && t >= h->dft_t0 && t < h->dft_t0 + (int64_t)h->dft_periods * h->T;
+}
+
 // Per-step arguments of the step from time tn to tn+1 reading population
 // buffer in and writing buffer out (a holds the common arguments).
 static void step_args_at(lbem_ctx *h, StepArgs &a, int64_t tn, int in, int out)
@@ -899,8 +905,7 @@ static void step_args_at(lbem_ctx *h, StepArgs &a, int64_t tn, int in, int out)
                 a.pw_wt[k] = make_float2((float)std::cos(ph), (float)std::sin(ph));
                 a.pw_t[k] = (float)ts;
             }
-        a.dft_on = (h->faces.nfaces > 0 && h->dft_t0 >= 1 && t >= h->dft_t0 &&
-                    t < h->dft_t0 + (int64_t)h->dft_periods * h->T);
+        a.dft_on = dft_at(h, t);
         if (a.dft_on) {
             const double ph = 2.0 * M_PI * (double)(t % h->T) / (double)h->T;
             a.dft_c = std::cos(ph);
@@ -1109,8 +1114,7 @@ static int march_pass(lbem_ctx *h, MarchArgs &m)
         LineMarch &l = m.line;
         for (int k = 0; k < K; ++k) {
             const int64_t t = n + 1 + k;
-            if (h->ms_n == 0 || h->dft_t0 < 1 || t < h->dft_t0 || t >= h->dft_t0 + (int64_t)h->dft_periods * h->T)
-                continue;
+            if (h->ms_n == 0 || !dft_at(h, t)) continue;
             const double ph = 2.0 * M_PI * (double)(t % h->T) / (double)h->T;
             const double c = std::cos(ph), s = std::sin(ph), sc = 2.0 / ((double)h->dft_periods * h->T);
             m.dft_mask |= 1u << k;
@@ -1164,8 +1168,8 @@ static int step_loop(lbem_ctx *h, int64_t n)
             continue;
         }
         // (a two-step pass stages the faces: where they are too large, single
-        // steps add to the accumulators in place)
-        if (pairs && n - k >= 2 && (h->xs_n > 0 || h->faces.nfaces == 0 || h->dft_t0 < 1)) {
+        // steps add to the accumulators in place while the window lasts)
+        if (pairs && n - k >= 2 && (h->xs_n > 0 || (!dft_at(h, h->t + 1) && !dft_at(h, h->t + 2)))) {
             // two steps in one pass: level n from f[cur], level n+2 into f[cur ^ 1]
             if (h->xs_cnt + 2 > kXBank) {
                 const int rc = flush_x_stage(h, true);

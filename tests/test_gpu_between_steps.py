@@ -84,3 +84,38 @@ def test_a_wave_injected_again_starts_from_an_empty_line(mode, shape, t):
         s.close()
     for a, b in zip(*got):
         assert np.isfinite(a).all() and np.array_equal(a, b)
+
+
+def test_two_step_passes_outside_the_window_of_faces_too_large_to_stage():
+    """A flat 3D grid whose NTFF faces (46 million cells) exceed what a pass can
+    stage takes single steps in the DFT window only: the kernels that run, and
+    the state and sums of a run through the window against single steps."""
+    import torch
+    from paper_2510_11042_gb300 import lbem
+    nx, ny, nz = 4800, 4800, 5
+    wave = W.PlaneWave(direction=(1.0, 0.0, 0.0), polarization=(0.0, 0.0, 1.0), wavelength=4.0, amplitude=1.0,
+                       ramp_periods=0.5, tf_lo=(6, 2, 1), tf_hi=(nx - 4, ny - 3, 3), ntff_lo=(5, 1, 0),
+                       ntff_hi=(nx - 3, ny - 2, 4), center=(nx / 2, ny / 2, 2.0), source_index=0)
+    eps = torch.ones((nz, ny, nx), device="cuda")
+    eps[:, :, 10:30] = 2.25
+    cells = [(x, y, z) for x in (4, 5, 6, 9, 12, 20) for y in (0, 1, 2, 77, 4799) for z in range(5)]
+    got = []
+    for fuse in (1, 2):
+        s = lbem.Solver((nx, ny, nz), eps, "3d", "f16")
+        s.set_step_fusion(fuse)
+        s.inject(wave)
+        s.set_dft_window(21, 1)
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            s.step(20)
+            s.sync()
+        names = [e.key for e in prof.key_averages()]
+        assert any("step2_kernel" in k for k in names) == (fuse == 2), names
+        s.step(15)
+        s.sync()
+        got.append([s.probe(cells), lbem.lbem_get_dft(s.h)[::97], s.incident_amplitude()])
+        s.close()
+        del s
+        torch.cuda.empty_cache()
+    assert np.abs(got[0][0]).max() > 0 and np.abs(got[0][1]).max() > 0
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
