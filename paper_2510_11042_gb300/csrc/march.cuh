@@ -302,6 +302,13 @@ template <int N> __device__ __forceinline__ void copy_async(uint32_t dst, const 
     else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(N) : "memory");
 }
 
+// A warp whose wait ran out: the error flag, then the end of its own copies.
+__device__ __forceinline__ void give_up(int *status, int lane)
+{
+    if (lane == 0) atomicOr(status, 1);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 template <class S>
 __device__ __forceinline__ void store_row(void *const *fout, int c, bool two, const Dir2<S> d[7])
 {

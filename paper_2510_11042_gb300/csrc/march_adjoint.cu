@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(32 * kRows, 1) march_adjoint_kernel(const __gr
 #pragma unroll 1
         for (int l = 0; l < K; ++l) {
             if (l > 0 && !await_rows(done, w, l, r - pa, r == pend)) {
-                if (lane == 0) atomicOr(a.status, 1);
+                give_up(a.status, lane);
                 return;
             }
             if (r >= y0 - (K - 1 - l) && r <= y1 - 1 + (K - 1 - l)) {
