@@ -34,6 +34,7 @@ struct lbem_ctx {
     float2 *pw_ph = nullptr;    // analytic source: per-axis phase factors, then 3 k_a (p - r0_a)
     float *pw_d = nullptr;
     bool mu_on = false;
+    bool maps_new = true;       // no step since 1/eps_r or 1/mu_r was written: the next one is not chained
     bool analytic = false;      // the plane wave is the closed-form source, not the line
     PlaneWaveA pw;
     float *line[kLineBufs] = {};  // incident line, line(t) in line[t mod kLineBufs]
@@ -325,6 +326,12 @@ static IncView inc_view(lbem_ctx *h)
     return v;
 }
 
+// Whether the next single step may chain to the kernel before it.
+static bool chain_steps(const lbem_ctx *h)
+{
+    return !h->maps_new && h->share == 1 && chain_pays(h->g.nx, h->g.ny, h->g.nz);
+}
+
 static void fill_common_args(lbem_ctx *h, StepArgs &a)
 {
     std::memset(&a, 0, sizeof a);
@@ -338,7 +345,7 @@ static void fill_common_args(lbem_ctx *h, StepArgs &a)
     a.scale = h->scale;
     a.inv_scale = h->inv_scale;
     a.status = h->flag + 1;
-    a.chain = h->share == 1 && chain_pays(a.nx, a.ny, a.nz);
+    a.chain = chain_steps(h);
     if (!h->has_wave) return;
     a.tfsf = h->analytic ? 2 : 1;
     a.line_on = h->analytic ? 0 : 1;
@@ -413,6 +420,7 @@ static int upload_inverse(lbem_ctx *h, const float *eps, int on_device, float *t
     CK(h, cudaMemcpyAsync(&bad, h->flag, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
     if (bad) return fail(h, LBEM_ERR_ARG, "%s must be finite and >= 1 in every cell", name);
+    h->maps_new = true;
     CK(h, launch_inv_eps(src, target, h->g.nx, h->g.ny, h->g.nz, h->nxp, h->flag, h->stream));
     h->launches += 1;
     return LBEM_OK;
@@ -542,6 +550,7 @@ int32_t lbem_set_permeability(lbem_handle h, const float *mu_r, int32_t mu_on_de
     h->adj_valid = false;
     if (!mu_r) {
         h->mu_on = false;
+        h->maps_new = true;
         CK(h, launch_fill(h->inv_mu, h->P, 1.0f, h->stream));
         return LBEM_OK;
     }
@@ -1011,6 +1020,7 @@ static LineRun line_run(lbem_ctx *h)
 static void march_common(lbem_ctx *h, MarchArgs &m)
 {
     std::memset(&m, 0, sizeof m);
+    m.chain = !h->maps_new;
     m.inv_eps = h->inv_eps;
     m.inv_mu = h->mu_on ? h->inv_mu : nullptr;
     m.status = h->flag + 1;
@@ -1151,12 +1161,12 @@ static int step_loop(lbem_ctx *h, int64_t n)
     if (pairs) fill_common_args(h, a2);
     MarchArgs m;
     if (march) march_common(h, m);
-    // The call's first step is launched plainly, behind whatever wrote the maps,
-    // the state and the line before; the others chain to the step before them.
-    const int chain = a.chain;
     for (int64_t k = 0; k < n;) {
-        a.chain = k > 0 ? chain : 0;
-        m.chain = k > 0;
+        if (k > 0 && h->maps_new) {
+            h->maps_new = false;
+            a.chain = chain_steps(h);
+            m.chain = 1;
+        }
         if (march && n - k >= kMarchSteps) {
             if (h->ms_cnt + kMarchSteps > h->ms_cap) {
                 const int rc = flush_march(h);
@@ -1233,6 +1243,7 @@ static int step_loop(lbem_ctx *h, int64_t n)
             if (rc != LBEM_OK) return rc;
         }
     }
+    if (n > 0) h->maps_new = false;
     const int rc = flush_march(h);
     if (rc != LBEM_OK) return rc;
     return flush_x_stage(h, false);  // every call leaves the DFT complete on the step stream
@@ -2250,7 +2261,6 @@ int32_t lbem_adjoint(lbem_handle h, const double *theta, const double *phi, cons
     StepArgs a;
     fill_common_args(h, a);
     a.dft_on = 0;
-    const int chain = a.chain;
     AdjointArgs b;
     std::memset(&b, 0, sizeof b);
     b.inv_eps = h->inv_eps;
@@ -2322,10 +2332,6 @@ int32_t lbem_adjoint(lbem_handle h, const double *theta, const double *phi, cons
         int64_t front = -1;
         for (int64_t k = 0; k < len;) {
             const int64_t t = t0 + k;   // state time before the step
-            // the sweep's first launch is plain, as lbem_step's
-            const bool behind = k > 0 || seg < L.nseg - 1;
-            a.chain = behind ? chain : 0;
-            m.chain = behind;
             if (march && len - k >= kMarchSteps) {
                 if (front != t + kMarchSteps) {
                     const int rc = march_line_start(h, m.line, rl, t, line_from(t + 1));

@@ -28,11 +28,12 @@ long long l2_bytes();
 // are visible.  Every kernel launched so calls chain_wait() before it touches
 // global memory that others write, and reads it by plain loads (the read-only path
 // is for data that does not change while the kernel lives); chain_release() lets
-// the next one be scheduled.  Exempt from the wait is what was complete before the
-// chain began: a chain's first kernel is launched plainly, in the call that builds
-// the chain, so 1/eps_r, 1/mu_r and the wave tables (step kernels), the angles and
-// the incident line's DFT (far_field_finalize), which no kernel of the chain
-// writes, may be read at any time.  us a step, plain -> chained: 200^2 with the
+// the next one be scheduled.  Exempt from the wait is what no kernel of the chain
+// writes and was complete before the chain began, with a plain launch: 1/eps_r and
+// 1/mu_r (the first step after a change of the maps is launched plainly) and the
+// wave tables (copied by a call that waits for them) in the step kernels, the angles
+// and the incident line's DFT in far_field_finalize (behind a plain launch of the
+// same call).  us a step, plain -> chained: 200^2 with the
 // closed-form source 6.2 -> 4.9 (3.2 with the source formed before the wait),
 // 520^2 HZ 4.7 -> 4.3, 64^3 FP32 12.5 -> 11.2, 512^2 adjoint 11.6 -> 10.5.
 template <class... P, class... A>
@@ -277,7 +278,7 @@ struct StepArgs {
     double *line_dft;          // [n_line][3][2]
     // reduced-precision storage: stored = population / scale (power of two)
     float scale, inv_scale;
-    int chain;                 // launch chained to the kernel before it, a step of the same call (launch_chained)
+    int chain;                 // launch chained to the kernel before it (launch_chained)
     // Tiles from the last to the first, on every other step: a step then starts
     // on the cells the one before it wrote last, which L2 (129 MB) still holds,
     // where the same order each time finds only evicted lines.  us a single step,
