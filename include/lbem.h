@@ -233,9 +233,10 @@ int32_t lbem_far_field(lbem_handle h, const double *theta_host, const double *ph
  * plus its edge halos in shared memory; it is taken where its blocks fill the
  * GPU (one wave of resident blocks).  In 2D a pass takes four steps, on every
  * grid of at least 2 x 2 cells: strips of 56 cells march along y with a row's
- * levels in registers.  Other grids, the closed-form source (bound by its
- * wave evaluations, not by memory), the steps a pass leaves over and handles
- * with in-place streaming take single steps.
+ * levels in registers; where the populations outgrow the L2 cache, two or three
+ * steps that are left over are a pass too.  Other grids, the closed-form source
+ * (bound by its wave evaluations, not by memory), the steps a pass leaves over
+ * and handles with in-place streaming take single steps.
  * 1 always takes single steps.  Anything else: LBEM_ERR_ARG. */
 int32_t lbem_set_step_fusion(lbem_handle h, int32_t steps_per_pass);
 

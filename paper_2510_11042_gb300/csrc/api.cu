@@ -974,6 +974,20 @@ static bool march_passes(const lbem_ctx *h)
     return h->fuse == 2 && !h->aa && !h->analytic && march_fits(h->g.mode, h->g.nx, h->g.ny, h->g.nz);
 }
 
+// Whether the two or three steps that 2D passes of kMarchSteps leave over (or
+// all that a call asks for) are a pass of their own: where the populations of the
+// grids stepping together outgrow L2.  In L2 a single step's second trip over
+// them is cheap, and the pass's launch for the line is not.  us a step, single
+// steps / passes, calls of two steps (of three): 1024^2 EZ FP16 (88 MB) 16.5 / 23.6
+// (16.5 / 17.4), 768^2 FP32 (99 MB) 12.4 / 12.3 (12.4 / 9.6), 850^2 FP32 (123 MB)
+// 16.6 / 17.2; 900^2 FP32 (140 MB) 18.9 / 16.5 (18.9 / 13.0), 1300^2 FP16 (143 MB)
+// 28.7 / 27.1 (28.8 / 22.0), 4096^2 FP32 410 / 226 (409 / 162), FP16 238 / 178 (238 /
+// 154).
+static bool short_passes(const lbem_ctx *h)
+{
+    return h->share * 2LL * h->Q * h->P * (long long)h->elem >= l2_bytes();
+}
+
 // Sum the staged 2D face fields into the DFT accumulators on the step stream.
 static int flush_march(lbem_ctx *h)
 {
@@ -1020,6 +1034,7 @@ static LineRun line_run(lbem_ctx *h)
 static void march_common(lbem_ctx *h, MarchArgs &m)
 {
     std::memset(&m, 0, sizeof m);
+    m.steps = kMarchSteps;
     m.chain = !h->maps_new;
     m.inv_eps = h->inv_eps;
     m.inv_mu = h->mu_on ? h->inv_mu : nullptr;
@@ -1064,19 +1079,19 @@ static void march_buffers(MarchArgs &m, const void *in, void *out, size_t plane_
         }
 }
 
-// The line's moments at the times n+1 .. n+K of a pass, from line(n+1), and
-// line(n+K): the start of a run of passes.
-static int march_line_start(lbem_ctx *h, const LineMarch &common, const LineRun &run, int64_t n, const float *from)
+// The line's moments at the times n+1 .. n+N of a pass of N steps, from
+// line(n+1), and line(n+N): the start of a run of passes.
+static int march_line_start(lbem_ctx *h, const LineMarch &common, const LineRun &run, int64_t n, int N,
+                            const float *from)
 {
-    constexpr int K = kMarchSteps;
     LineMarch st = common;
     st.dft_mask = 0;
     st.from = from;
-    st.steps = K - 1;
+    st.steps = N - 1;
     st.lm_from = run.moments(n + 1);
-    for (int k = 0; k < K; ++k) {
+    for (int k = 0; k < N - 1; ++k) {
         st.lm[k] = run.moments(n + 2 + k);
-        st.full[k] = k == K - 2 ? run.at(n + K) : nullptr;
+        st.full[k] = k == N - 2 ? run.at(n + N) : nullptr;
         source_fields(h, n + 2 + k, st.src_E[k], st.src_H[k]);
     }
     CK(h, launch_line_start(h->g.mode, st, h->stream));
@@ -1084,45 +1099,46 @@ static int march_line_start(lbem_ctx *h, const LineMarch &common, const LineRun 
     return LBEM_OK;
 }
 
-// The line's part of the pass from time n: the moments it reads, and the
-// line's steps n+K+1 .. n+2K for the next pass.
-static void march_line(lbem_ctx *h, MarchArgs &m, const LineRun &run, int64_t n)
+// The line's part of a pass of N steps from time n: the moments it reads, and
+// the line's steps n+N+1 .. n+N+K for a next pass of K.
+static void march_line(lbem_ctx *h, MarchArgs &m, const LineRun &run, int64_t n, int N)
 {
     constexpr int K = kMarchSteps;
     LineMarch &l = m.line;
-    l.from = run.at(n + K);
+    l.from = run.at(n + N);
     l.steps = K;
     l.dft_mask = 0;
     for (int k = 0; k < K; ++k) {
-        const int64_t tl = n + K + 1 + k;
-        m.lm[k] = l.lm_now[k] = run.moments(n + 1 + k);
+        const int64_t tl = n + N + 1 + k;
+        m.lm[k] = l.lm_now[k] = k < N ? run.moments(n + 1 + k) : nullptr;
         l.lm[k] = run.moments(tl);
         l.full[k] = (k == 0 || k == K - 1) ? run.at(tl) : nullptr;
         source_fields(h, tl, l.src_E[k], l.src_H[k]);
     }
 }
 
-// kMarchSteps steps in one pass: level n from f[cur] to f[cur ^ 1].  The pass
-// needs the line's moments at its own times and advances the line for the
-// next one; where the previous pass did not (a first pass, or single steps
-// since), a small launch starts it.
-static int march_pass(lbem_ctx *h, MarchArgs &m)
+// N steps in one pass: level n from f[cur] to f[cur ^ 1].  The pass needs the
+// line's moments at its own times and advances the line for a next one of K;
+// where the previous pass did not (a first pass, single steps since, or another
+// number of steps now), a small launch starts it.
+static int march_pass(lbem_ctx *h, MarchArgs &m, int N)
 {
     constexpr int K = kMarchSteps;
     const int64_t n = h->t;
     const int cnt0 = h->ms_cnt;
+    m.steps = N;
     march_buffers(m, h->f[h->cur], h->f[h->cur ^ 1], (size_t)h->P * h->elem);
     m.dft_mask = 0;
     if (h->has_wave) {
         const LineRun run = line_run(h);
-        if (h->line_front != n + K) {
-            const int rc = march_line_start(h, m.line, run, n, line_at(h, n + 1));
+        if (h->line_front != n + N) {
+            const int rc = march_line_start(h, m.line, run, n, N, line_at(h, n + 1));
             if (rc != LBEM_OK) return rc;
-            h->line_front = n + K;
+            h->line_front = n + N;
         }
-        march_line(h, m, run, n);
+        march_line(h, m, run, n, N);
         LineMarch &l = m.line;
-        for (int k = 0; k < K; ++k) {
+        for (int k = 0; k < N; ++k) {
             const int64_t t = n + 1 + k;
             if (h->ms_n == 0 || !dft_at(h, t)) continue;
             const double ph = 2.0 * M_PI * (double)(t % h->T) / (double)h->T;
@@ -1144,9 +1160,9 @@ static int march_pass(lbem_ctx *h, MarchArgs &m)
         return cuda_fail(h, e, "2D pass launch");
     }
     h->launches += 1;
-    if (h->has_wave) h->line_front = n + 2 * K;
+    if (h->has_wave) h->line_front = n + N + K;
     h->cur ^= 1;
-    h->t += K;
+    h->t += N;
     return LBEM_OK;
 }
 
@@ -1156,7 +1172,7 @@ static int step_loop(lbem_ctx *h, int64_t n)
 {
     StepArgs a;
     fill_common_args(h, a);
-    const bool pairs = two_step_passes(h), march = march_passes(h);
+    const bool pairs = two_step_passes(h), march = march_passes(h), few = march && short_passes(h);
     StepArgs a2;
     if (pairs) fill_common_args(h, a2);
     MarchArgs m;
@@ -1167,14 +1183,15 @@ static int step_loop(lbem_ctx *h, int64_t n)
             a.chain = chain_steps(h);
             m.chain = 1;
         }
-        if (march && n - k >= kMarchSteps) {
+        if (march && n - k >= (few ? 2 : kMarchSteps)) {
             if (h->ms_cnt + kMarchSteps > h->ms_cap) {
                 const int rc = flush_march(h);
                 if (rc != LBEM_OK) return rc;
             }
-            const int rc = march_pass(h, m);
+            const int N = (int)std::min<int64_t>(n - k, kMarchSteps);
+            const int rc = march_pass(h, m, N);
             if (rc != LBEM_OK) return rc;
-            k += kMarchSteps;
+            k += N;
             continue;
         }
         // (a two-step pass stages the faces: where they are too large, single
@@ -2334,11 +2351,11 @@ int32_t lbem_adjoint(lbem_handle h, const double *theta, const double *phi, cons
             const int64_t t = t0 + k;   // state time before the step
             if (march && len - k >= kMarchSteps) {
                 if (front != t + kMarchSteps) {
-                    const int rc = march_line_start(h, m.line, rl, t, line_from(t + 1));
+                    const int rc = march_line_start(h, m.line, rl, t, kMarchSteps, line_from(t + 1));
                     if (rc != LBEM_OK) return rc;
                 }
                 march_buffers(m, state, rf[into], plane_bytes);
-                march_line(h, m, rl, t);
+                march_line(h, m, rl, t, kMarchSteps);
                 for (int j = 0; j < kMarchSteps; ++j) m.rec[j] = rec + (size_t)(k + j) * NE * h->P;
                 const cudaError_t e = launch_march(h->g.mode, h->g.storage, m, true, 1, h->stream);
                 if (e != cudaSuccess) return cuda_fail(h, e, "replay pass launch");

@@ -14,8 +14,8 @@ namespace lbem {
 
 constexpr int kMaxDevices = 64;  // per-device set-up caches
 // Buffers of the incident line, line(t) in buffer t mod kLineBufs: a 2D pass
-// from time n to n + 4 reads line(n+4) and writes line(n+5) and line(n+8),
-// after which line(n+4), line(n+5) and line(n+8) are in use.
+// from time n to n + N reads line(n+N) and writes line(n+N+1) and line(n+N+4),
+// after which these three are in use.
 constexpr int kLineBufs = 5;
 // Streaming multiprocessors and L2 bytes of the current device (queried once
 // per device; 0 if the query fails).
@@ -395,10 +395,12 @@ struct LineMarch {
     const float *lm_now[kMarchSteps];
 };
 
-// One pass of kMarchSteps steps from time n (times n + 1 + k below).
+// One pass of `steps` steps (kMarchSteps, or two or three) from time n (times
+// n + 1 + k below).
 struct MarchArgs {
+    int steps;
     const void *fin[14];           // per direction: the pair groups, the singles of level n
-    void *fout[14];                // the same of level n + kMarchSteps
+    void *fout[14];                // the same of level n + steps
     const float *inv_eps, *inv_mu; // inv_mu: NULL without a mu_r map
     int *status;                   // kernel error flags (bit 0: a bounded wait ran out)
     int nx, ny, nxp;

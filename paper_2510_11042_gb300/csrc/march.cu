@@ -16,7 +16,11 @@
 //     A chunk recomputes up to three rows on each side.
 //   * The next row's level n is copied into shared memory (cp.async) while the
 //     warp is at the row before.
-// Level n is read from memory and level n+4 written once per four steps.
+// Level n is read from memory and level n+4 written once per four steps.  Passes
+// of two or three steps take what a call of few steps asks for, on large grids
+// (short_passes in api.cu): the same kernel with fewer levels and the same strips.
+// (Strips of 60 cells, which two levels would allow, start off the sectors' ends:
+// 2048^2 EZ FP16 51 -> 54 us a step, 250 x 8000 FP16 34 -> 38; 3000^2 gained 7 %.)
 //
 // Every sum, product and rounding is that of update_cell (step_cell.cuh), two
 // cells to a packed FP32x2 instruction; 16-bit storage rounds the levels between
@@ -309,7 +313,8 @@ template <int MODE> __global__ void __launch_bounds__(32) line_start_kernel(cons
     line_march<MODE>(l, blockIdx.x);
 }
 
-template <int MODE, class S, bool MU, bool REC>
+// A pass of N steps.
+template <int MODE, class S, bool MU, bool REC, int N>
 __global__ void __launch_bounds__(32 * kRows, 16 / kRows) march_kernel(const __grid_constant__ MarchArgs a)
 {
     using Y = YBuf<S>;
@@ -329,7 +334,7 @@ __global__ void __launch_bounds__(32 * kRows, 16 / kRows) march_kernel(const __g
     const int xc = min(max(cx.x, 0), a.nxp - 2);  // loads stay inside the row
     // owned rows [y0, y1); level n+1 runs over [pa, pend]
     const int y0 = chunk * a.rows, y1 = min(a.ny, y0 + a.rows);
-    const int pa = max(y0 - (K - 1), 0), pend = min(y1 - 1 + (K - 1), a.ny - 1);
+    const int pa = max(y0 - (N - 1), 0), pend = min(y1 - 1 + (N - 1), a.ny - 1);
     __shared__ __align__(8) unsigned long long done[kRows][K];
     init_rows(done);
     chain_wait();
@@ -355,12 +360,12 @@ __global__ void __launch_bounds__(32 * kRows, 16 / kRows) march_kernel(const __g
             row.special = __any_sync(kAll, diel || min(cx.dmin, min(r, a.ny - 1 - r)) < a.w);
         }
 #pragma unroll 1
-        for (int l = 0; l < K; ++l) {
-            if (l > 0 && !await_rows(done, w, l, r - pa, r == pend)) {
+        for (int l = 0; l < N; ++l) {
+            if (l > 0 && !await_rows(done, w, l, r - pa, r == pend, N)) {
                 give_up(a.status, lane);
                 return;
             }
-            if (r >= y0 - (K - 1 - l) && r <= y1 - 1 + (K - 1 - l)) {
+            if (r >= y0 - (N - 1 - l) && r <= y1 - 1 + (N - 1 - l)) {
                 from_left<S>(d[1], ends);
                 from_right<S>(d[2], ends);
                 if (l > 0) {
@@ -374,7 +379,11 @@ __global__ void __launch_bounds__(32 * kRows, 16 / kRows) march_kernel(const __g
                 update2<MODE, MU, REC>(a, f, l, cx, row, ie, im);
 #pragma unroll
                 for (int i = 0; i < 7; ++i) d[i] = to_dir<S>(f + 3 * i);
-                if (l < K - 1) {
+                if (N == 2 && l == 0 && !await_slot(done, w, r - pa)) {
+                    give_up(a.status, lane);
+                    return;
+                }
+                if (l < N - 1) {
                     Y::put(Y::at(ybuf, w, l, 0), lane, d[3]);
                     Y::put(Y::at(ybuf, w, l, 1), lane, d[4]);
                 } else if (cx.own) {
@@ -414,10 +423,10 @@ __global__ void __launch_bounds__(128) dft_flush_2d_kernel(const __grid_constant
 
 // ---- host side
 std::mutex g_march_mu;
-int g_march_bps[kMaxDevices][2][3][2][2];
+int g_march_bps[kMaxDevices][2][3][2][2][K + 1];
 template <class S> constexpr int storage_slot() { return std::is_same<S, float>::value ? 0 : (std::is_same<S, __half>::value ? 1 : 2); }
 
-template <int MODE, class S, bool MU, bool REC>
+template <int MODE, class S, bool MU, bool REC, int N>
 cudaError_t launch_march_t(MarchArgs a, int share, cudaStream_t s)
 {
     int dev = 0, bps = 0;
@@ -426,32 +435,47 @@ cudaError_t launch_march_t(MarchArgs a, int share, cudaStream_t s)
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     {
         std::lock_guard<std::mutex> lock(g_march_mu);
-        int &n = g_march_bps[dev][MODE][storage_slot<S>()][MU][REC];
-        e = march_setup_kernel(march_kernel<MODE, S, MU, REC>, march_smem<S, MU>(), n);
+        int &got = g_march_bps[dev][MODE][storage_slot<S>()][MU][REC][N];
+        e = march_setup_kernel(march_kernel<MODE, S, MU, REC, N>, march_smem<S, MU>(), got);
         if (e != cudaSuccess) return e;
-        bps = n;
+        bps = got;
     }
     a.strips = (a.nx + kStrip - 1) / kStrip;
-    a.rows = march_rows(a.ny, a.strips, std::max<long long>(1, (long long)std::max(1, sm_count()) * bps / share));
+    a.rows = march_rows(a.ny, a.strips, std::max<long long>(1, (long long)std::max(1, sm_count()) * bps / share), N == 2);
     const long long chunks = (a.ny + a.rows - 1) / a.rows;
     a.line_warps = a.line.steps > 0 ? line_march_warps(a.line) : 0;
     a.line_blocks = (a.line_warps + kRows - 1) / kRows;
     const long long blocks = a.line_blocks + chunks * a.strips;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    return launch_chained(a.chain != 0 && share == 1, march_kernel<MODE, S, MU, REC>, (unsigned)blocks, 32 * kRows, march_smem<S, MU>(), s, a);
+    return launch_chained(a.chain != 0 && share == 1, march_kernel<MODE, S, MU, REC, N>, (unsigned)blocks, 32 * kRows, march_smem<S, MU>(), s, a);
+}
+
+template <int MODE, class S, bool MU>
+cudaError_t launch_march_steps(bool rec, const MarchArgs &a, int share, cudaStream_t s)
+{
+    static_assert(K == 4, "one case each");
+    if constexpr (std::is_same<S, float>::value && !MU) {
+        if (rec && a.steps == K) return launch_march_t<MODE, S, MU, true, K>(a, share, s);
+    }
+    if (rec) return cudaErrorInvalidValue;
+    switch (a.steps) {
+    case 2: return launch_march_t<MODE, S, MU, false, 2>(a, share, s);
+    case 3: return launch_march_t<MODE, S, MU, false, 3>(a, share, s);
+    case K: return launch_march_t<MODE, S, MU, false, K>(a, share, s);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 template <int MODE>
 cudaError_t launch_march_mode(int storage, bool mu, bool rec, const MarchArgs &a, int share, cudaStream_t s)
 {
-    if (rec) return storage == 0 && !mu ? launch_march_t<MODE, float, false, true>(a, share, s) : cudaErrorInvalidValue;
     switch (storage * 2 + (mu ? 1 : 0)) {
-    case 0: return launch_march_t<MODE, float, false, false>(a, share, s);
-    case 1: return launch_march_t<MODE, float, true, false>(a, share, s);
-    case 2: return launch_march_t<MODE, __half, false, false>(a, share, s);
-    case 3: return launch_march_t<MODE, __half, true, false>(a, share, s);
-    case 4: return launch_march_t<MODE, __nv_bfloat16, false, false>(a, share, s);
-    case 5: return launch_march_t<MODE, __nv_bfloat16, true, false>(a, share, s);
+    case 0: return launch_march_steps<MODE, float, false>(rec, a, share, s);
+    case 1: return launch_march_steps<MODE, float, true>(rec, a, share, s);
+    case 2: return launch_march_steps<MODE, __half, false>(rec, a, share, s);
+    case 3: return launch_march_steps<MODE, __half, true>(rec, a, share, s);
+    case 4: return launch_march_steps<MODE, __nv_bfloat16, false>(rec, a, share, s);
+    case 5: return launch_march_steps<MODE, __nv_bfloat16, true>(rec, a, share, s);
     default: return cudaErrorInvalidValue;
     }
 }

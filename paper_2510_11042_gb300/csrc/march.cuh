@@ -270,22 +270,34 @@ __device__ __forceinline__ Ends make_ends(int strip, const Cols &c, int nx)
 }
 
 // The waits of level l > 0 of row r (index i of the chunk's, the last one with
-// last set): level l - 1 of the rows above and below.  The same waits (also
-// where the level itself is not computed, in the chunk's first and last rows)
-// keep the groups of row r until both neighbours have read them: row r + kRows,
-// which takes their place, starts once row r is finished, so both have read its
-// first two levels; and it reaches the third once the rows beside it are under
-// way, whose warps have then finished the rows beside r.  The last row, which
-// has none below it, waits for the row kRows - 1 before it in that one's stead.
+// last set) in a pass of n levels: level l - 1 of the rows above and below.  The
+// same waits (also where the level itself is not computed, in the chunk's first
+// and last rows) keep the groups of row r until both neighbours have read them:
+// row r + kRows, which takes their place, starts once row r is finished, so both
+// have read its groups but those of level n - 2; and it reaches that level once
+// the rows beside it are under way, whose warps have then finished the rows beside
+// r.  (With two levels it is the first one, which has no waits of its own:
+// await_slot.)  The last row, which has none below it, waits for the row kRows - 1
+// before it in that one's stead.
 // A wait tells a phase only from its neighbours, so no warp may wait for a
 // slot's second row before the slot's first has begun: the block barrier.
-__device__ __forceinline__ bool await_rows(unsigned long long (*done)[K], int w, int l, int i, bool last)
+__device__ __forceinline__ bool await_rows(unsigned long long (*done)[K], int w, int l, int i, bool last, int n)
 {
     const int above = w == 0 ? kRows - 1 : w - 1, below = w == kRows - 1 ? 0 : w + 1;
     if (l == 1 && i < kRows) block_sync();
     bool ok = i == 0 || await(&done[above][l - 1], (uint32_t)(i - 1) / kRows);
     if (!last) ok = ok && await(&done[below][l - 1], (uint32_t)(i + 1) / kRows);
-    else if (i >= kRows - 1) ok = ok && await(&done[below][K - 1], (uint32_t)(i - (kRows - 1)) / kRows);
+    else if (i >= kRows - 1) ok = ok && await(&done[below][n - 1], (uint32_t)(i - (kRows - 1)) / kRows);
+    return __all_sync(kAll, ok);
+}
+// The wait of a row's first level in a pass of two, before its groups are
+// written: the rows beside the one whose place they take (i - kRows) are finished.
+__device__ __forceinline__ bool await_slot(unsigned long long (*done)[K], int w, int i)
+{
+    if (i < kRows) return true;
+    const int above = w == 0 ? kRows - 1 : w - 1, below = w == kRows - 1 ? 0 : w + 1;
+    const bool ok = (i == kRows || await(&done[above][1], (uint32_t)(i - kRows - 1) / kRows)) &&
+                    await(&done[below][1], (uint32_t)(i - kRows + 1) / kRows);
     return __all_sync(kAll, ok);
 }
 __device__ __forceinline__ void init_rows(unsigned long long (*done)[K])
@@ -348,9 +360,12 @@ __device__ __forceinline__ void store_row(void *const *fout, int c, bool two, co
 // 19.3 -> 17.1 ms.  The count that is best without it stays where it costs less than
 // 3 % more: there several waves measured between 10 % slower (1024^2: 12.2 in one
 // wave, 13.5 in two) and no better (3400^2: 90.6 in five, 92.5 in seven).
-constexpr double kSlowest = 0.18, kStay = 1.03;
-inline int march_rows(int ny, int strips, long long cap)
+// Passes of two levels, which have the least work to a byte, like shorter chunks
+// still (4096^2 EZ with kSlowest -> kSlowestTwo: FP16 186 -> 178, FP32 240 -> 226).
+constexpr double kSlowest = 0.18, kSlowestTwo = 0.6, kStay = 1.03;
+inline int march_rows(int ny, int strips, long long cap, bool two = false)
 {
+    const double slowest = two ? kSlowestTwo : kSlowest;
     struct Plan { long long chunks; double waves, rows; } plain = {0, 0, 0}, best = {0, 0, 0};
     auto cost = [](const Plan &p, double extra) { return (p.waves + extra) * (p.rows + 12.0); };
     for (long long w = 1; w <= 256; ++w) {
@@ -359,10 +374,10 @@ inline int march_rows(int ny, int strips, long long cap)
         const long long n = (ny + rows - 1) / rows;
         const Plan p = {n, (double)((n * strips + cap - 1) / cap), (double)rows};
         if (plain.chunks == 0 || cost(p, 0.0) < cost(plain, 0.0)) plain = p;
-        if (best.chunks == 0 || cost(p, kSlowest) < cost(best, kSlowest)) best = p;
+        if (best.chunks == 0 || cost(p, slowest) < cost(best, slowest)) best = p;
         if (rows <= kMarchMinRows) break;
     }
-    const long long chunks = (cost(plain, kSlowest) < kStay * cost(best, kSlowest) ? plain : best).chunks;
+    const long long chunks = (cost(plain, slowest) < kStay * cost(best, slowest) ? plain : best).chunks;
     return (int)std::max<long long>((ny + chunks - 1) / chunks, kMarchMinRows);
 }
 

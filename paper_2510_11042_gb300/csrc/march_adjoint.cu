@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(32 * kRows, 1) march_adjoint_kernel(const __gr
         row.face = r >= a.nt_lo[1] && r <= a.nt_hi[1] && (cx.xface || r == a.nt_lo[1] || r == a.nt_hi[1]);
 #pragma unroll 1
         for (int l = 0; l < K; ++l) {
-            if (l > 0 && !await_rows(done, w, l, r - pa, r == pend)) {
+            if (l > 0 && !await_rows(done, w, l, r - pa, r == pend, K)) {
                 give_up(a.status, lane);
                 return;
             }
