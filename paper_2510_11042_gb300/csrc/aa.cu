@@ -110,7 +110,11 @@ __device__ __forceinline__ void aa_store_dir(void *const *b, int k, void *fb, in
 // for: these kernels wait on their loads, and what serves them best depends on
 // how the compiler schedules these around the update (300^3 in the DFT window,
 // us a step, [late, 7 / 8 blocks; early, 7 / 8]: BF16 [876 / 814; 876 / 850],
-// FP16 [849 / 847; 820 / 839], FP32 [1464 / 1360; 1369 / 1360]).
+// FP16 [849 / 847; 820 / 839], FP32 [1464 / 1360; 1369 / 1360]).  The same ones are
+// best from 96^3 to 450^3 (as chosen; early, 8; early, 7): BF16 19.6; 19.7; 19.6 at
+// 96^3, 237; 247; 256 at 200^3, 2565; 2652; 2754 at 450^3, FP16 18.1; 18.6; 18.2,
+// 237; 245; 237 and 2564; 2642; 2564, FP32 36.2; 36.2; 37.1, 401; 401; 408 and 4570;
+// 4570; 4620.
 template <class S> __host__ __device__ constexpr bool aa_late() { return std::is_same<S, __nv_bfloat16>::value; }
 template <int MODE, class S, bool ANA> constexpr int aa_blocks()
 {
@@ -284,7 +288,7 @@ constexpr int kAaBX = 128;  // threads per block at most (row_threads)
 template <int MODE, class S, bool MU, bool ANA, int KIND>
 cudaError_t launch_aa_t(StepArgs a, const AaArgs &g, cudaStream_t s)
 {
-    const int tx = row_threads(a.nx);
+    const int tx = row_threads(a.nx, (long long)a.ny * a.nz);
     a.nblk_x = (a.nx + tx - 1) / tx;
     a.rows_per_block = 1;
     const long long blocks = (long long)a.nblk_x * a.ny * a.nz;

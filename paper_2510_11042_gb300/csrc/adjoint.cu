@@ -329,7 +329,7 @@ __global__ void adjoint_finalize_kernel(const double *grad, const float *inv_eps
 template <int MODE>
 cudaError_t launch_adj(AdjointArgs a, cudaStream_t s)
 {
-    const int tx = row_threads(a.nx);
+    const int tx = row_threads(a.nx, (long long)a.ny * a.nz);
     a.nblk_x = (a.nx + tx - 1) / tx;
     const long long blocks = (long long)a.nblk_x * a.ny * a.nz;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;

@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kFlushThreads, 16) dft_flush_x_kernel(const Df
 template <int MODE, class S, bool REC = false, bool MU = false, bool ANA = false>
 cudaError_t launch_cell(StepArgs a, cudaStream_t s)
 {
-    const int tx = row_threads(a.nx);
+    const int tx = row_threads(a.nx, (long long)a.ny * a.nz);
     a.nblk_x = (a.nx + tx - 1) / tx;
     a.rows_per_block = rows_of<S>();
     const bool direct = MODE == 2 && a.dft_on && !a.xstage;  // the faces are too large to stage
