@@ -109,6 +109,15 @@ __device__ __forceinline__ void row_cells(const StepArgs &a, int bx, int y, int 
 // closed-form source (ANA) also holds the source terms and takes 96 (5 blocks:
 // 2.83 ms at 384^3, against 3.98 ms spilling at 7).  These were chosen by timing
 // the 384^3 sphere and 256^2 to 4096^2 EZ grids on GB300.
+// BF16 rows of four, without a mu_r map, are compiled for 8 blocks (64 registers,
+// 36 bytes spilled): us a step, 7 blocks -> 8: 96^3 27.7 -> 24.9, 200^3 238 -> 214, 300^3
+// 735 -> 703, 384^3 1465 -> 1409; with a map (300^3 767 -> 814), one row a block (64^3
+// 6.60 -> 6.72) and in FP16 7 stay.
+template <int MODE, class S, bool MU, bool ANA, bool ONE> __host__ __device__ constexpr int step_blocks()
+{
+    if (MODE == 2 && ANA) return 5;
+    return MODE == 2 && std::is_same<S, __nv_bfloat16>::value && !MU && !ANA && !ONE ? 8 : 7;
+}
 template <class S> __host__ __device__ constexpr int rows_of() { return sizeof(S) == 4 ? 2 : 4; }
 
 // Whether the kernel loads through the read-only path, and so is never chained.
@@ -116,7 +125,7 @@ template <class S, bool ONE> __host__ __device__ constexpr bool read_only_path()
 
 template <int MODE, class S, int BX, bool REC = false, bool MU = false, bool ANA = false, bool ONE = false,
           int FORM = kStaged>
-__global__ void __launch_bounds__(BX, (ANA && MODE == 2) ? 5 : 7) step_kernel_cell(const StepArgs a)
+__global__ void __launch_bounds__(BX, (step_blocks<MODE, S, MU, ANA, ONE>())) step_kernel_cell(const StepArgs a)
 {
     constexpr int R = ONE ? 1 : rows_of<S>();
     constexpr bool WAIT = ANA && ONE && MODE != 2;
