@@ -126,7 +126,7 @@ template <int MODE, class S, bool ANA> constexpr int aa_blocks()
 // where the scheme puts direction i: the push step writes direction i through
 // fout_q (aimed at slot opp(i)) and the in-place step reads it through fin_q
 // (aimed at slot opp(i)).
-template <int MODE, class S, int BX, bool MU, bool ANA, int KIND, int FORM>
+template <int MODE, class S, bool MU, bool ANA, int KIND, int FORM>
 __device__ __forceinline__ void aa_row(const StepArgs &a, const AaArgs &g, int bx, int y, int z)
 {
     constexpr int Q = Planes<MODE>::Q;
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(BX, (aa_blocks<MODE, S, ANA>())) aa_step_kerne
     }
     const int tile = a.flip ? a.nblk_main - 1 - b : b;
     const int r = tile / a.nblk_x;
-    aa_row<MODE, S, BX, MU, ANA, KIND, FORM>(a, g, tile % a.nblk_x, r % a.ny, r / a.ny);
+    aa_row<MODE, S, MU, ANA, KIND, FORM>(a, g, tile % a.nblk_x, r % a.ny, r / a.ny);
 }
 
 // The face cell k of axis ax (the other two coordinates, the lower one

@@ -67,7 +67,7 @@ namespace {
 // evaluations above all, comes before the wait for the kernel before this one
 // (chain_wait): 200^2 EZ 4.9 -> 3.2 us a step.  In 3D the terms' registers beside
 // 42 populations would spill.
-template <int MODE, class S, int BX, bool REC = false, bool MU = false, bool ANA = false, int FORM = kStaged,
+template <int MODE, class S, bool REC = false, bool MU = false, bool ANA = false, int FORM = kStaged,
           bool NCL = false, bool WAIT = false>
 __device__ __forceinline__ void row_cells(const StepArgs &a, int bx, int y, int z)
 {
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(BX, (step_blocks<MODE, S, MU, ANA, ONE>())) st
     const int r0 = (tile / a.nblk_x) * R;
     const int r1 = min(r0 + R, a.ny * a.nz);
     for (int r = r0; r < r1; ++r)
-        row_cells<MODE, S, BX, REC, MU, ANA, FORM, read_only_path<S, ONE>(), WAIT>(a, bx, r % a.ny, r / a.ny);
+        row_cells<MODE, S, REC, MU, ANA, FORM, read_only_path<S, ONE>(), WAIT>(a, bx, r % a.ny, r / a.ny);
 }
 
 constexpr int kBX = 128;  // threads per block at most; cells per row tile of the batched kernel
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(kBX) batch_kernel(const BatchArgs b)
                 const int r0 = (li / sa.nblk_x) * b.rows_per_item;
                 const int bx = li % sa.nblk_x;
                 for (int r = r0; r < min(r0 + b.rows_per_item, rows); ++r)
-                    row_cells<MODE, S, kBX, false, false, false, kDirect>(sa, bx, r % sa.ny, r / sa.ny);
+                    row_cells<MODE, S, false, false, false, kDirect>(sa, bx, r % sa.ny, r / sa.ny);
             }
             __syncthreads();
         }
