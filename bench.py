@@ -60,18 +60,29 @@ def b_cell(mode: str, storage: str) -> int:
 
 
 def kernel_source_hash(two_d: bool = False) -> str:
-    """Hash of the step kernels' source: in 3D step.cu, step2.cu, step_cell.cuh
-    and the StepArgs definition, in 2D march.cu and march.cuh."""
+    """Hash of what makes the step kernels: in 3D step.cu, step2.cu, step_cell.cuh
+    and the StepArgs definition, in 2D march.cu, march.cuh, step_cell.cuh, the
+    kMarch constants and the LineMarch and MarchArgs definitions."""
     csrc = os.path.join(ROOT, "paper_2510_11042_gb300", "csrc")
     h = hashlib.sha256()
-    for name in ("march.cu", "march.cuh") if two_d else ("step.cu", "step2.cu", "step_cell.cuh"):
+    for name in ("march.cu", "march.cuh", "step_cell.cuh") if two_d else ("step.cu", "step2.cu", "step_cell.cuh"):
         with open(os.path.join(csrc, name), "rb") as fh:
             h.update(fh.read())
-    if not two_d:
-        hdr = open(os.path.join(csrc, "lbem_internal.cuh")).read()
-        i = hdr.index("struct StepArgs {")
+    with open(os.path.join(csrc, "lbem_internal.cuh")) as fh:
+        hdr = fh.read()
+    for name in ("LineMarch", "MarchArgs") if two_d else ("StepArgs",):
+        i = hdr.index(f"struct {name} {{")
         h.update(hdr[i:hdr.index("};", i)].encode())
+    if two_d:
+        h.update("\n".join(line for line in hdr.splitlines() if "constexpr" in line and " kMarch" in line).encode())
     return h.hexdigest()[:16]
+
+
+def updates_per_pass(mode: str, fusion: int) -> int:
+    """Lattice updates of one pass of lbem_step on a grid that takes passes
+    (fusion 2, as lbem_get_step_fusion reports it), four in 2D and two in 3D;
+    1 on one that takes single steps."""
+    return fusion if fusion == 1 or mode == "3d" else 4
 
 
 def traffic_from_profile(workload: str, storage: str):
@@ -484,8 +495,8 @@ def run_probe_2d(dev, n=4096, updates=60):
     """Step throughput of the 2D EZ path on a grid well above L2 (4096^2 x 21
     populations, 2.8 GB in FP32): a cylinder of the cylinder workload's
     proportions, CUDA events around `updates` lattice updates, with the pass
-    lbem_step takes by default (four updates per pass) and with single steps.  hbm_frac is the byte model
-    (B_cell per update) over the time per update."""
+    lbem_step takes by default (four updates per pass) and with single steps.
+    hbm_frac is the byte model (B_cell per update) over the time per update."""
     import torch
     from paper_2510_11042_gb300 import lbem
     p = W.cylinder_problem(n=n, x=5.0, wavelength=40.0, eps_in=2.25, w=20, mode="ez", periods=1)
@@ -509,16 +520,17 @@ def run_probe_2d(dev, n=4096, updates=60):
             gbs = bc * n * n / (ms / 1e3) / 1e9
             rec[fuse] = {"kernel_ms": round(ms, 4), "mlups": round(n * n / (ms / 1e3) / 1e6, 1),
                          "bytes_per_cell": bc, "achieved_gbs": round(gbs, 1), "hbm_frac": round(gbs / hbm, 4),
-                         "steps_per_pass": s.step_fusion()}
+                         "steps_per_pass": updates_per_pass("ez", s.step_fusion())}
             s.close()
             del s
             torch.cuda.empty_cache()
         out[st] = dict(rec[2], single_step=rec[1], speedup_vs_single_step=round(rec[1]["kernel_ms"] /
                                                                                 rec[2]["kernel_ms"], 3))
         # the four-step kernel's own DRAM traffic (ncu, committed summary), over the time of its launch
-        traffic = traffic_from_profile(f"cylinder_{n}_ez", st) if rec[2]["steps_per_pass"] == 2 else None
+        per = rec[2]["steps_per_pass"]
+        traffic = traffic_from_profile(f"cylinder_{n}_ez", st) if per > 1 else None
         if traffic:
-            gbs_t = traffic / (4 * rec[2]["kernel_ms"] / 1e3) / 1e9
+            gbs_t = traffic / (per * rec[2]["kernel_ms"] / 1e3) / 1e9
             out[st]["dram_traffic_per_launch"] = traffic
             out[st]["dram_traffic_gbs"] = round(gbs_t, 1)
             out[st]["dram_traffic_frac"] = round(gbs_t / hbm, 4)
@@ -559,7 +571,7 @@ def run_cylinder_1024(dev, updates=120):
             working = (2 * (42 if mode == "3d" else 21) * (4 if st == "f32" else 2) + 4) * cells
             out[f"{mode}_{st}"] = {"kernel_ms": round(ms, 4), "mlups": round(cells / (ms / 1e3) / 1e6, 1),
                                    "bytes_per_cell": bc, "achieved_gbs": round(gbs, 1),
-                                   "hbm_frac": round(gbs / hbm, 4), "steps_per_pass": s.step_fusion(),
+                                   "hbm_frac": round(gbs / hbm, 4), "steps_per_pass": updates_per_pass(mode, s.step_fusion()),
                                    "working_set_mb": round(working / 1e6, 1),
                                    "label": ("L2-assisted" if l2 and working < 3 * l2 else "HBM")}
             s.close()
