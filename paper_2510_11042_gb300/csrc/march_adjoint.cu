@@ -11,8 +11,9 @@
 // over the four levels; the recorded D of the four steps is copied with the row.
 //
 // Bound as the forward pass on small grids: instruction issue and the rows'
-// waits.  512^2 EZ, us a step: backward, one launch a step 8.3 -> 6.3, replay
-// (march_kernel with the recorded D) 8.3 -> 5.2.
+// waits.  512^2 EZ, us a step: backward, one launch a step 8.3 -> 6.3, and 5.5
+// chained to the launch before; replay (march_kernel with the recorded D) 8.3 -> 5.2,
+// and 4.6.
 #include <algorithm>
 #include <cstring>
 #include <mutex>

@@ -36,7 +36,7 @@
 // proportional to the scattered field rather than to the incident one.
 //
 // The incident line (same update, eps_r = 1, absorbing layer at both ends,
-// hard source) runs one step ahead of the lattice in three rotating buffers:
+// hard source) runs one step ahead of the lattice in rotating buffers (kLineBufs):
 // during step n the lattice reads line(n+1) and the first blocks of the same
 // launch write line(n+2).
 //

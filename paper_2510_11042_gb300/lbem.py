@@ -606,14 +606,17 @@ class Solver:
         return lbem_far_field(self.h, theta, phi, with_amplitudes)
 
     def set_step_fusion(self, steps_per_pass):
-        """2 (default): two steps per pass over the populations where they pay
-        (grids of any mode and storage, with or without a mu_r map, that fill
-        the GPU; not the closed-form source or in-place streaming); 1: single
-        steps."""
+        """2 (default): several steps per pass over the populations, any storage,
+        with or without a mu_r map: four in 2D (and the two or three that are
+        left over where the populations outgrow L2), two in 3D on grids that
+        fill the GPU; not with the closed-form source or in-place streaming.
+        1: single steps."""
         lbem_set_step_fusion(self.h, steps_per_pass)
 
     def step_fusion(self):
-        """The steps per pass lbem_step takes as the handle is configured now."""
+        """2 where lbem_step takes several steps per pass as the handle is
+        configured now (four in 2D, two in 3D), else 1: the value
+        set_step_fusion takes."""
         return lbem_get_step_fusion(self.h)
 
     def set_far_field_precision(self, precision):
